@@ -388,7 +388,7 @@ typedef struct epbr_mesh {
 } epbr_mesh;
 
 /* Device workspace epbr_raster_gbuffer needs: 8 B per pixel (nearest (depth, triangle) key),
- * 64 B and 8 B per triangle (set-up, item offsets), each part 256-byte aligned. */
+ * 64 B and 8 B per triangle (set-up, queue entry), each part 256-byte aligned. */
 epbr_status epbr_raster_workspace_size(int32_t num_triangles, int32_t width, int32_t height, size_t* bytes);
 
 /* Writes the FP32 G-buffer `out` (rt[0] albedo + metal, rt[1] normal + rough, rt[3] eye depth;
@@ -408,9 +408,9 @@ epbr_status epbr_raster_gbuffer(const epbr_mesh* mesh, const epbr_camera* camera
                                 const epbr_gbuffer* out, int32_t* ids, int64_t ids_pitch, void* workspace,
                                 size_t workspace_bytes, void* stream);
 
-/* Device workspace epbr_shadow_maps needs for maps of size x size texels: the key images and
- * triangle set-ups of up to 8 lights at a time (8 x (8 B per texel + 72 B per triangle), about
- * 130 MB for 512^2 maps of a 200,000-triangle mesh), reused group after group. */
+/* Device workspace epbr_shadow_maps needs for maps of size x size texels: 8 x (8 B per texel + 72 B
+ * per triangle), about 130 MB for 512^2 maps of a 200,000-triangle mesh, which holds the triangle
+ * set-ups of at least 8 lights at a time, reused group after group. */
 epbr_status epbr_shadow_maps_workspace_size(int32_t num_triangles, int32_t size, size_t* bytes);
 
 /* Shadow maps by rendering the mesh "only as a depth map" from each light as from a normal
@@ -419,8 +419,8 @@ epbr_status epbr_shadow_maps_workspace_size(int32_t num_triangles, int32_t size,
  * writes for that camera (same coverage, depth and tie rules; +inf where nothing is drawn).
  * `maps` is DEVICE float[num_maps][S][S] (dense rows), the layout epbr_shadows.maps takes; the
  * cameras are host structs (the world -> light-view rows epbr_shadows.cameras holds for shading
- * are the inverse of each camera's view_to_world).  Up to 8 lights are rendered by one set of
- * launches (set-up, scan, coverage, depth), groups one after the other through `workspace`
+ * are the inverse of each camera's view_to_world).  8 to 32 lights (as many as
+ * `workspace` has room for) are rendered by one set of launches, groups one after the other through it
  * (DEVICE, 256-byte aligned, epbr_shadow_maps_workspace_size bytes), stream-ordered; no
  * allocation.  EPBR_ERR_UNSUPPORTED above 2^28 triangles.  Re-render when the scene or a light
  * moves. */
