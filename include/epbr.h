@@ -438,9 +438,8 @@ typedef struct epbr_surfels {
   int32_t reserved;
 } epbr_surfels;
 
-/* Device workspace epbr_surfel_gbuffer needs: 40 B per pixel (nearest depth, nine attribute
- * sums), 4 B per pixel column and row (pixel rays), 96 B and 8 B per surfel (set-up, task
- * offsets), each part 256-byte aligned. */
+/* Device workspace epbr_surfel_gbuffer needs: 40 B per pixel, 4 B per pixel column and row, 96 B
+ * and 8 B per surfel (list entries of the cells it covers, pixel box), each part 256-byte aligned. */
 epbr_status epbr_surfel_workspace_size(int32_t num_surfels, int32_t width, int32_t height, size_t* bytes);
 
 /* Writes the FP32 G-buffer `out` (rt[0] albedo + metal, rt[1] normal + rough, rt[3] eye depth;
@@ -454,7 +453,7 @@ epbr_status epbr_surfel_workspace_size(int32_t num_surfels, int32_t width, int32
  * s <= depth * (1 + depth_tolerance) adds its albedo, unit normal, metal and rough with weight 1,
  * and the G-buffer holds their means (the normal renormalised).  These decisions are evaluated in
  * FP32 with every product, sum, quotient and square root rounded, in a fixed order, so they are
- * reproducible bit for bit; the sums are float atomics (their order varies).  `weight` (DEVICE
+ * reproducible bit for bit; the order of the sums varies.  `weight` (DEVICE
  * float, NULL allowed, rows of weight_pitch bytes) receives the number of blended surfels, 0 for
  * background.  `workspace` DEVICE, 256-byte aligned, at least epbr_surfel_workspace_size bytes.
  * Stream-ordered; no allocation. */
