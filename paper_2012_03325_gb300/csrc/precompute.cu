@@ -1,8 +1,8 @@
 // Image-based lighting precompute (paper Sec. 3.1; split sum of Karis 2013):
 //   k_brdf_lut          BRDF integration table (A, B), one warp per texel, Kahan + shuffles
-//   k_irradiance_part   exact-quadrature irradiance, per-block partial sums over a slice of
-//                       source texels staged in shared memory (packed FP32x2 over output pairs,
-//                       plain sums per staged tile, Kahan across tiles)
+//   k_irradiance_part   exact-quadrature irradiance, per-block partial sums over a slice of source
+//                       row pieces: a row's hemisphere is one interval of columns, summed from
+//                       sums of 64 and 8 texels and single texels at its ends (Kahan across pieces)
 //   k_irradiance_final  one warp per output: lanes sum the block partials, a shuffle butterfly
 //                       adds the lanes (fixed order: deterministic), then the ratio
 //   k_prefilter         GGX-prefiltered levels 1..M-1, one block per row of a level: the row's
@@ -77,9 +77,9 @@ __global__ void k_brdf_lut(int S, int N, float2* __restrict__ lut) {
 // ------------------------------------------------------------------------------------------
 // Irradiance: sum_t L_t max(n.d_t, 0) Omega_t / sum_t max(n.d_t, 0) Omega_t
 // ------------------------------------------------------------------------------------------
-constexpr int kIrrThreads = 128;
-constexpr int kIrrOutPerThread = 4;  // outputs per thread and pass (two packed pairs): 512 per pass
-constexpr int kIrrTile = 256;        // source texels staged per step
+constexpr int kIrrThreads = 512;     // threads per block at most, an output each
+constexpr int kIrrPiece = 2048;      // source columns staged per step
+constexpr int kIrrGroup = 8, kIrrSeg = 64;  // columns per sum of the two levels
 constexpr int kIrrTexelsPerBlock = 1024;
 constexpr int kIrrMaxBlocks = 608;
 
@@ -101,83 +101,188 @@ __device__ __forceinline__ float3 texel_dir(int i, int j, int W, int H) {
   return f3(st * sp, ct, -st * cp);
 }
 
-// Each block sums over its slice of source texels for every output texel; a thread owns
-// kIrrOutPerThread outputs as two pairs whose arithmetic runs in packed FP32x2 instructions.
-// A source texel is staged once per tile as d Omega (max(n.d, 0) Omega = max(n.(d Omega), 0) since
-// Omega > 0) and L, every value duplicated into both halves of a pair: (dx, dx, dy, dy),
-// (dz, dz, Lr, Lr), (Lg, Lg, Lb, Lb).  Per tile the four sums of each output (L w and w) are
-// plain FP32; the tile's sums are then added to the slice totals with Kahan compensation.
+// With the azimuth phi of source column x and of the output, n.d = A cos(phi_x - phi_i) + B, A and B
+// constant along a source row, so that the hemisphere of n is one interval of the row's columns
+// (none, some or all), and over any columns inside it
+//   sum L (n.d) = A (cos phi_i sum L cos phi_x + sin phi_i sum L sin phi_x) + B sum L.
+// Sums of these three over 8 and over 64 columns are formed once per row piece, so that an output
+// needs about 30 terms per row instead of all its texels; the texels at the interval's ends are
+// clamped one by one, as the definition has it.
+struct IrrSums {
+  float t[3], c[3], s[3];  // sums of L, L cos phi, L sin phi (three channels)
+  float c1, s1, pad;       // sums of cos phi, sin phi
+};
+
+struct IrrAcc {
+  float r = 0.0f, g = 0.0f, b = 0.0f, w = 0.0f;
+};
+
+__device__ __forceinline__ void irr_add(IrrAcc& a, const IrrSums& q, float ac, float as, float B, float n) {
+  a.r += fmaf(ac, q.c[0], fmaf(as, q.s[0], B * q.t[0]));
+  a.g += fmaf(ac, q.c[1], fmaf(as, q.s[1], B * q.t[1]));
+  a.b += fmaf(ac, q.c[2], fmaf(as, q.s[2], B * q.t[2]));
+  a.w += fmaf(ac, q.c1, fmaf(as, q.s1, B * n));
+}
+
+// Shared memory of a piece of n columns, one entry skipped per segment: the outputs of a warp, a
+// segment apart on the usual maps, then read different banks.
+__host__ __device__ inline int irr_at(int column) { return column + column / kIrrSeg; }
+__host__ __device__ inline int irr_group_at(int g) { return g + g / (kIrrSeg / kIrrGroup); }
+struct IrrShared {
+  float4* texel;
+  IrrSums* group;
+  IrrSums* seg;
+  float2* phi;  // cos, sin of the columns' azimuths
+  size_t bytes;
+};
+__host__ __device__ inline IrrShared irr_shared(char* base, int n) {
+  IrrShared s;
+  size_t off = 0;
+  s.texel = (float4*)base;
+  off += sizeof(float4) * (irr_at(n - 1) + 1);
+  s.group = (IrrSums*)(base + off);
+  off += sizeof(IrrSums) * (irr_group_at(n / kIrrGroup) + 1);
+  s.seg = (IrrSums*)(base + off);
+  off += sizeof(IrrSums) * (n / kIrrSeg + 1);
+  s.phi = (float2*)(base + off);
+  s.bytes = off + sizeof(float2) * (irr_at(n - 1) + 1);
+  return s;
+}
+
+// Bound by issue (the terms of every output and row): 39 us for a 2048 x 1024 environment, 319 us
+// when every output summed every source texel in packed FP32x2 arithmetic (62% of the FMA pipe).
+// Each block takes the row pieces of its slice, a thread one output per pass (blockIdx.y and its
+// stride: the passes).  A piece's sums (L w and w, with the row's solid angle) are added to the
+// slice totals with Kahan compensation.  ROUND: a piece is a whole row of whole segments, so the
+// interval is walked round the row's end and every output of a row has the same count of terms.
+template <bool ROUND>
 __global__ void __launch_bounds__(kIrrThreads) k_irradiance_part(const float4* __restrict__ env, int We,
                                                                  int He, int Wi, int Hi,
                                                                  float4* __restrict__ part) {
-  __shared__ float4 s_src[kIrrTile][3];
-  long long ntex = (long long)We * He;
-  long long per = (ntex + gridDim.x - 1) / gridDim.x;
-  long long t0 = per * blockIdx.x;
-  long long t1 = t0 + per < ntex ? t0 + per : ntex;
-  int nout = Wi * Hi;
+  extern __shared__ __align__(16) char s_irr[];
+  const IrrShared sh = irr_shared(s_irr, min(We, kIrrPiece));
+  const int tid = threadIdx.x, threads = blockDim.x;
+  const int per_row = (We + kIrrPiece - 1) / kIrrPiece;
+  const long long pieces = (long long)He * per_row;
+  const long long p0 = pieces * blockIdx.x / gridDim.x, p1 = pieces * (blockIdx.x + 1) / gridDim.x;
+  const int nout = Wi * Hi;
+  constexpr int kPer = kIrrSeg / kIrrGroup;
   // Omega of row y = (2 pi / W)(cos(pi y / H) - cos(pi (y + 1) / H))
   //               = (4 pi / W) sin(pi (y + 0.5) / H) sin(pi / (2 H))   (product form)
-  float row_k = 4.0f * kPi / We * sinpif(0.5f / He);
-  for (int og = 0; og < nout; og += kIrrThreads * kIrrOutPerThread) {
-    // pair p holds outputs og + (2p + h) * kIrrThreads + tid, h = 0, 1; an absent output has n = 0
-    float2 nx[2], ny[2], nz[2];
-#pragma unroll
-    for (int p = 0; p < 2; ++p) {
-      float3 a, b;
-      int oa = og + (2 * p) * kIrrThreads + threadIdx.x, ob = oa + kIrrThreads;
-      a = oa < nout ? texel_dir(oa % Wi, oa / Wi, Wi, Hi) : f3(0, 0, 0);
-      b = ob < nout ? texel_dir(ob % Wi, ob / Wi, Wi, Hi) : f3(0, 0, 0);
-      nx[p] = make_float2(a.x, b.x), ny[p] = make_float2(a.y, b.y), nz[p] = make_float2(a.z, b.z);
-    }
-    Kahan acc[kIrrOutPerThread][4];
-    for (long long base = t0; base < t1; base += kIrrTile) {
-      int cnt = (int)(t1 - base < kIrrTile ? t1 - base : kIrrTile);
+  const float row_k = 4.0f * kPi / We * sinpif(0.5f / He);
+  for (int og = blockIdx.y * threads; og < nout; og += gridDim.y * threads) {
+    const int o = og + tid, i = min(o, nout - 1) % Wi, j = min(o, nout - 1) / Wi;
+    float st, ct, sp, cp;
+    sincospif((j + 0.5f) / Hi, &st, &ct);
+    sincospif(2.0f * ((i + 0.5f) / Wi) - 1.0f, &sp, &cp);
+    const float X = (i + 0.5f) * ((float)We / (float)Wi) - 0.5f;  // the output's azimuth as a source column
+    Kahan acc[4];
+    int have = -1;  // the piece of a row whose azimuths are staged
+    for (long long p = p0; p < p1; ++p) {
+      const int y = (int)(p / per_row), c = (int)(p - (long long)y * per_row);
+      const int c0 = c * kIrrPiece, n = min(kIrrPiece, We - c0);
       __syncthreads();
-      for (int q = threadIdx.x; q < cnt; q += kIrrThreads) {
-        long long t = base + q;
-        int x = (int)(t % We), y = (int)(t / We);
-        float3 d = texel_dir(x, y, We, He) * (row_k * sinpif((y + 0.5f) / He));
-        float4 L = __ldg(env + t);
-        s_src[q][0] = make_float4(d.x, d.x, d.y, d.y);
-        s_src[q][1] = make_float4(d.z, d.z, L.x, L.x);
-        s_src[q][2] = make_float4(L.y, L.y, L.z, L.z);
-      }
-      __syncthreads();
-      float2 sr[2], sg[2], sb[2], sw[2];
-#pragma unroll
-      for (int p = 0; p < 2; ++p) sr[p] = sg[p] = sb[p] = sw[p] = make_float2(0.0f, 0.0f);
-#pragma unroll 4
-      for (int q = 0; q < cnt; ++q) {
-        const float4 u = s_src[q][0], v = s_src[q][1], z = s_src[q][2];
-        const float2 dx = make_float2(u.x, u.y), dy = make_float2(u.z, u.w), dz = make_float2(v.x, v.y);
-        const float2 Lr = make_float2(v.z, v.w), Lg = make_float2(z.x, z.y), Lb = make_float2(z.z, z.w);
-#pragma unroll
-        for (int p = 0; p < 2; ++p) {
-          float2 w = __ffma2_rn(nx[p], dx, __ffma2_rn(ny[p], dy, __fmul2_rn(nz[p], dz)));
-          w = make_float2(fmaxf(w.x, 0.0f), fmaxf(w.y, 0.0f));
-          sr[p] = __ffma2_rn(Lr, w, sr[p]);
-          sg[p] = __ffma2_rn(Lg, w, sg[p]);
-          sb[p] = __ffma2_rn(Lb, w, sb[p]);
-          sw[p] = __fadd2_rn(sw[p], w);
+      for (int q = tid; q < n; q += threads) {
+        sh.texel[irr_at(q)] = __ldg(env + (long long)y * We + c0 + q);
+        if (have != c) {
+          float sx, cx;
+          sincospif(2.0f * ((c0 + q + 0.5f) / We) - 1.0f, &sx, &cx);
+          sh.phi[irr_at(q)] = make_float2(cx, sx);
         }
       }
+      have = c;
+      __syncthreads();
+      for (int g = tid; g < n / kIrrGroup; g += threads) {
+        IrrSums q = {};
 #pragma unroll
-      for (int p = 0; p < 2; ++p) {
-        acc[2 * p][0].add(sr[p].x), acc[2 * p][1].add(sg[p].x), acc[2 * p][2].add(sb[p].x);
-        acc[2 * p][3].add(sw[p].x);
-        acc[2 * p + 1][0].add(sr[p].y), acc[2 * p + 1][1].add(sg[p].y), acc[2 * p + 1][2].add(sb[p].y);
-        acc[2 * p + 1][3].add(sw[p].y);
+        for (int k = 0; k < kIrrGroup; ++k) {
+          // the lanes of a warp start at different texels of their groups: fewer bank conflicts
+          const int at = irr_at(g * kIrrGroup + ((k + tid) & (kIrrGroup - 1)));
+          const float4 L = sh.texel[at];
+          const float2 f = sh.phi[at];
+          const float v[3] = {L.x, L.y, L.z};
+#pragma unroll
+          for (int h = 0; h < 3; ++h) {
+            q.t[h] += v[h];
+            q.c[h] = fmaf(v[h], f.x, q.c[h]);
+            q.s[h] = fmaf(v[h], f.y, q.s[h]);
+          }
+          q.c1 += f.x;
+          q.s1 += f.y;
+        }
+        sh.group[irr_group_at(g)] = q;
       }
-    }
+      __syncthreads();
+      constexpr int kWords = sizeof(IrrSums) / 4;
+      for (int q = tid; q < n / kIrrSeg * kWords; q += threads) {
+        const int g = q / kWords, f = q - g * kWords;
+        float sum = 0.0f;
 #pragma unroll
-    for (int r = 0; r < kIrrOutPerThread; ++r) {
-      int o = og + r * kIrrThreads + threadIdx.x;
-      if (o < nout)
-        part[(size_t)blockIdx.x * nout + o] =
-            make_float4(acc[r][0].s - acc[r][0].c, acc[r][1].s - acc[r][1].c,
-                        acc[r][2].s - acc[r][2].c, acc[r][3].s - acc[r][3].c);
+        for (int k = 0; k < kPer; ++k) sum += ((const float*)&sh.group[irr_group_at(g * kPer + k)])[f];
+        ((float*)&sh.seg[g])[f] = sum;
+      }
+      __syncthreads();
+      float sty, cty;
+      sincospif((y + 0.5f) / He, &sty, &cty);
+      const float omega = row_k * sty;
+      const float A = st * sty, B = ct * cty, ac = A * cp, as = A * sp;
+      if (!(B > -A)) continue;  // the row lies below the horizon
+      // columns lo .. hi (modulo We) hold every texel with n.d > 0, at most a rounding beyond
+      int lo = 0, hi = We - 1;
+      const bool all = !(B < A);
+      if (!all) {
+        const float D = acosf(-B / A) * (We * kInv2Pi);
+        lo = (int)ceilf(X - D) - 1;
+        hi = min((int)floorf(X + D) + 1, lo + We - 1);  // once round: a gap of one column is lo itself
+      }
+      IrrAcc a;
+      auto wrap = [We](int q, int period) { return ROUND && q >= period ? q - period : q; };
+      // whole groups strictly inside lo .. hi (not the two columns at either end, whose texels are
+      // clamped), whole segments where they fit; columns from .. to - 1 of the piece
+      auto interval = [&](int x0, int x1, int i0, int i1) {
+        const int g0 = (i0 + kIrrGroup - 1) / kIrrGroup, g1 = max(i1, 0) / kIrrGroup;
+        const int s0 = (g0 + kPer - 1) / kPer, s1 = g1 / kPer;
+        const bool groups = g0 < g1, segs = groups && s0 < s1;
+        // single texels x0 .. e0 - 1 and b1 .. x1 - 1, groups g0 .. h0 - 1 and h1 .. g1 - 1
+        const int e0 = groups ? g0 * kIrrGroup : x1, b1 = groups ? g1 * kIrrGroup : x1;
+        const int h0 = segs ? s0 * kPer : g1, h1 = segs ? s1 * kPer : g1;
+        const int nt = (e0 - x0) + (x1 - b1), ng = groups ? (h0 - g0) + (g1 - h1) : 0, nx = segs ? s1 - s0 : 0;
+        for (int k = 0, q = x0; k < nt; ++k, ++q) {
+          if (q == e0) q = b1;
+          const int at = irr_at(wrap(q, We));
+          const float2 f = sh.phi[at];
+          const float4 L = sh.texel[at];
+          const float w = fmaxf(fmaf(ac, f.x, fmaf(as, f.y, B)), 0.0f);
+          a.r = fmaf(L.x, w, a.r);
+          a.g = fmaf(L.y, w, a.g);
+          a.b = fmaf(L.z, w, a.b);
+          a.w += w;
+        }
+        for (int k = 0, q = g0; k < ng; ++k, ++q) {
+          if (q == h0) q = h1;
+          irr_add(a, sh.group[irr_group_at(wrap(q, We / kIrrGroup))], ac, as, B, (float)kIrrGroup);
+        }
+        for (int k = 0; k < nx; ++k) irr_add(a, sh.seg[wrap(s0 + k, We / kIrrSeg)], ac, as, B, (float)kIrrSeg);
+      };
+      if (ROUND) {
+        if (lo < 0) lo += We, hi += We;
+        interval(lo, hi + 1, all ? lo : lo + 2, all ? hi + 1 : hi - 1);
+      } else {
+#pragma unroll 1
+        for (int turn = -1; turn <= 1; ++turn) {  // the interval's copies one turn apart
+          const int l = lo + turn * We - c0, h = hi + turn * We - c0;
+          const int x0 = max(l, 0), x1 = min(h, n - 1) + 1;
+          if (x0 < x1) interval(x0, x1, !all && l > -2 ? l + 2 : 0, min(!all && h < n + 1 ? h - 1 : n, n));
+        }
+      }
+      acc[0].add(a.r * omega);
+      acc[1].add(a.g * omega);
+      acc[2].add(a.b * omega);
+      acc[3].add(a.w * omega);
     }
+    if (o < nout)
+      part[(size_t)blockIdx.x * nout + o] =
+          make_float4(acc[0].s - acc[0].c, acc[1].s - acc[1].c, acc[2].s - acc[2].c, acc[3].s - acc[3].c);
   }
 }
 
@@ -508,6 +613,32 @@ extern "C" epbr_status epbr_precompute_ibl_workspace_size(const epbr_ibl_params*
   return ok();
 }
 
+namespace epbr {
+
+// Partial sums into `ws` (at least irr_workspace_bytes), then the outputs.
+static epbr_status launch_irradiance(const epbr_env* env, int Wi, int Hi, float4* ws, float4* out, cudaStream_t s) {
+  const int We = env->width, He = env->height, nout = Wi * Hi;
+  const bool round = We <= kIrrPiece && We % kIrrSeg == 0;
+  // slices of whole row pieces, as even as the three blocks an SM holds allow
+  const long long pieces = (long long)He * ((We + kIrrPiece - 1) / kIrrPiece), room = 3LL * num_sms();
+  const long long each = (pieces + room - 1) / room;
+  const int nb = (int)std::min<long long>(irr_blocks(We, He), (pieces + each - 1) / each);
+  // few slices (a small environment): smaller blocks, several per slice
+  const int threads = nb >= num_sms() ? kIrrThreads : 128, passes = (nout + threads - 1) / threads;
+  const int gy = (int)std::min<long long>(std::min(passes, 65535), std::max<long long>(1, room / nb));
+  const size_t smem = irr_shared(nullptr, std::min(We, kIrrPiece)).bytes;
+  void (*k)(const float4*, int, int, int, int, float4*) = round ? k_irradiance_part<true> : k_irradiance_part<false>;
+  if (smem > 48 * 1024 && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    return fail(EPBR_ERR_CUDA, "irradiance: shared-memory attribute: %s", cudaGetErrorString(cudaGetLastError()));
+  k<<<dim3(nb, gy), threads, smem, s>>>((const float4*)env->texels, We, He, Wi, Hi, ws);
+  epbr_status st = check_launch("k_irradiance_part");
+  if (st) return st;
+  k_irradiance_final<<<(unsigned)(((long long)nout * 32 + 255) / 256), 256, 0, s>>>(ws, nb, nout, out);
+  return check_launch("k_irradiance_final");
+}
+
+}  // namespace epbr
+
 extern "C" epbr_status epbr_irradiance(const epbr_env* env, int32_t Wi, int32_t Hi, float* out,
                                        void* ws, size_t ws_bytes, void* stream) {
   epbr_status st = validate_env(env);
@@ -519,15 +650,7 @@ extern "C" epbr_status epbr_irradiance(const epbr_env* env, int32_t Wi, int32_t 
   if (!ws || ws_bytes < need || (uintptr_t)ws % 16)
     return fail(EPBR_ERR_NO_MEMORY, "irradiance: workspace needs %zu bytes (16-byte aligned), got %zu", need,
                 ws ? ws_bytes : (size_t)0);
-  int nb = irr_blocks(env->width, env->height);
-  cudaStream_t s = (cudaStream_t)stream;
-  k_irradiance_part<<<nb, kIrrThreads, 0, s>>>((const float4*)env->texels, env->width, env->height, Wi,
-                                               Hi, (float4*)ws);
-  if ((st = check_launch("k_irradiance_part"))) return st;
-  int nout = Wi * Hi;
-  k_irradiance_final<<<(unsigned)(((long long)nout * 32 + 255) / 256), 256, 0, s>>>((const float4*)ws, nb, nout,
-                                                                                   (float4*)out);
-  if ((st = check_launch("k_irradiance_final"))) return st;
+  if ((st = launch_irradiance(env, Wi, Hi, (float4*)ws, (float4*)out, (cudaStream_t)stream))) return st;
   return ok();
 }
 
@@ -619,17 +742,9 @@ extern "C" epbr_status epbr_irradiance_noalloc(const epbr_env* env, int32_t Wi, 
                 Wi, Hi, env->width, env->height, need, kStaticScratchBytes);
   void* ws = nullptr;
   if ((st = static_scratch(&ws))) return st;
-  int nb = irr_blocks(env->width, env->height);
-  cudaStream_t s = (cudaStream_t)stream;
   // Every partial the final pass reads is written by the first pass, so the scratch needs no
   // clearing between calls.
-  k_irradiance_part<<<nb, kIrrThreads, 0, s>>>((const float4*)env->texels, env->width, env->height, Wi, Hi,
-                                               (float4*)ws);
-  if ((st = check_launch("k_irradiance_part"))) return st;
-  int nout = Wi * Hi;
-  k_irradiance_final<<<(unsigned)(((long long)nout * 32 + 255) / 256), 256, 0, s>>>((const float4*)ws, nb, nout,
-                                                                                   (float4*)out);
-  if ((st = check_launch("k_irradiance_final"))) return st;
+  if ((st = launch_irradiance(env, Wi, Hi, (float4*)ws, (float4*)out, (cudaStream_t)stream))) return st;
   return ok();
 }
 
