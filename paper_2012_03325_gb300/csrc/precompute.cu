@@ -5,9 +5,11 @@
 //                       sums of 64 and 8 texels and single texels at its ends (Kahan across pieces)
 //   k_irradiance_final  one warp per output: lanes sum the block partials, a shuffle butterfly
 //                       adds the lanes (fixed order: deterministic), then the ratio
-//   k_prefilter         GGX-prefiltered levels 1..M-1, one block per row of a level: the row's
-//                       sample geometry computed once (the sampling frame turns with the texel
-//                       about the pole axis), each texel sums its samples at shifted columns
+//   k_prefilter_rows    GGX-prefiltered levels 1 and 2 of the usual maps, one block per row of a level:
+//                       the row's sample geometry computed once (the sampling frame turns with the
+//                       texel about the pole axis), each texel sums its samples at shifted columns of
+//                       source rows staged in shared memory
+//   k_prefilter         the other levels, source rows read through L1
 #include <cuda.h>  // CUcontext and CUresult for the context queries (fetched at run time)
 
 #include <algorithm>
@@ -313,8 +315,7 @@ __global__ void k_irradiance_final(const float4* __restrict__ part, int nblocks,
 // ------------------------------------------------------------------------------------------
 struct ChainDev {
   int M;
-  int nlev;                       // levels written: 1..M-1
-  long long off[EPBR_MAX_LEVELS + 1];  // texel prefix sums over levels 1..M-1
+  int first;  // the first level a launch writes
   int W[EPBR_MAX_LEVELS], H[EPBR_MAX_LEVELS];
   float4* dst[EPBR_MAX_LEVELS];
 };
@@ -353,53 +354,45 @@ __device__ __forceinline__ float2 prefilter_src_xy(float3 l, int W0, int H0) {
   return make_float2(fmaf(u, (float)W0, -0.5f), fmaf(v, (float)H0, -0.5f));
 }
 
-// Per kept sample, for texel 0 of the row, in order of source row: INT_SHIFT (W0 a multiple of
-// Wm) stores the four bilinear weights times n.l and (column, row); otherwise the two row weights
-// times n.l and the source x coordinate (the column fraction then varies along the row), and the
-// row.  Samples are visited in order of their source row so that consecutive samples read the
-// same two rows, which stay in L1 (a deterministic bitonic sort of (row, sample) keys).
-template <bool INT_SHIFT>
-__global__ void __launch_bounds__(kPrefilterThreads) k_prefilter(MapDev src, ChainDev ch, int N) {
-  // dynamic shared memory: N float4 weights, N int2 (column, row), N ushort sorted positions; the
-  // sort keys ((source row << 16) | kept-sample index, N unsigned) occupy the weights' space
-  // until the records are written
-  extern __shared__ __align__(16) float4 s_pf[];
-  __shared__ int s_base[kPrefilterMaxSamples / 32 + 1];
-  __shared__ float s_wsum[kPrefilterThreads / 32];
-  float4* s_w = s_pf;
-  int2* s_xy = (int2*)(s_pf + N);
-  unsigned short* s_pos = (unsigned short*)(s_xy + N);
-  unsigned* s_key = (unsigned*)s_pf;
-  const int m = blockIdx.y + 1;
-  const int W = ch.W[m], H = ch.H[m];
-  const int segs = (W + kPrefilterSeg - 1) / kPrefilterSeg;
-  const int j = blockIdx.x / segs, i0 = (blockIdx.x - j * segs) * kPrefilterSeg;
-  if (j >= H) return;  // block-uniform
-  const int W0 = src.W, H0 = src.H;
-  const float r = (float)m / (float)(ch.M - 1);
+// Shared memory of a block that prefilters a row: N float4 weights, N int2, N ushort sorted
+// positions; the sort keys (N unsigned) occupy the weights' space until the records are written.
+struct PrefilterShared {
+  int base[kPrefilterMaxSamples / 32 + 1];
+  float wsum[16];
+};
+
+// The samples of row j of level m as records in order of source row (a deterministic bitonic sort of
+// (source row + 1, sample) keys), by a block of THREADS threads.  `keyed(keys, ns)` sees the sorted
+// keys, `emit(position, sample (.z = n.l), source x, y for texel 0)` writes a record.  Returns the
+// number of kept samples and their weight sum sum_k n.l_k (the same for every texel of the level).
+template <int THREADS, typename Keyed, typename Emit>
+__device__ __forceinline__ int prefilter_records(PrefilterShared& sh, unsigned* s_key, unsigned short* s_pos, int m,
+                                                 int M, int j, int W, int H, int W0, int H0, int N, float& wsum,
+                                                 Keyed keyed, Emit emit) {
+  const float r = (float)m / (float)(M - 1);
   const float a2 = r * r * r * r;
   const float invN = 1.0f / N;
   const int groups = (N + 31) / 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // kept samples per group of 32, then an exclusive prefix over the groups (sample order)
-  for (int gi = warp; gi < groups; gi += kPrefilterThreads / 32) {
+  for (int gi = warp; gi < groups; gi += THREADS / 32) {
     int sidx = gi * 32 + lane;
     bool keep = sidx < N && prefilter_sample(sidx, a2, invN).z > 0.0f;
     unsigned bal = __ballot_sync(0xffffffffu, keep);
-    if (lane == 0) s_base[gi] = __popc(bal);
+    if (lane == 0) sh.base[gi] = __popc(bal);
   }
   __syncthreads();
   if (tid == 0) {
     int acc = 0;
     for (int gi = 0; gi < groups; ++gi) {
-      int c = s_base[gi];
-      s_base[gi] = acc;
+      int c = sh.base[gi];
+      sh.base[gi] = acc;
       acc += c;
     }
-    s_base[groups] = acc;
+    sh.base[groups] = acc;
   }
   __syncthreads();
-  const int ns = s_base[groups];
+  const int ns = sh.base[groups];
   // the frame of texel 0 of the row: n, T = y x n / |y x n| = (-cos phi0, 0, -sin phi0), B = n x T
   const float3 n = texel_dir(0, j, W, H);
   float sp0, cp0;
@@ -407,25 +400,25 @@ __global__ void __launch_bounds__(kPrefilterThreads) k_prefilter(MapDev src, Cha
   const float3 T = f3(-cp0, 0.0f, -sp0);
   const float3 B = cross3(n, T);
   // pass A: each kept sample's source row, as a sort key
-  for (int gi = warp; gi < groups; gi += kPrefilterThreads / 32) {
+  for (int gi = warp; gi < groups; gi += THREADS / 32) {
     int sidx = gi * 32 + lane;
     float4 e = sidx < N ? prefilter_sample(sidx, a2, invN) : make_float4(0, 0, 0, 0);
     bool keep = sidx < N && e.z > 0.0f;
     unsigned bal = __ballot_sync(0xffffffffu, keep);
     if (keep) {
-      const int q = s_base[gi] + __popc(bal & ((1u << lane) - 1u));
+      const int q = sh.base[gi] + __popc(bal & ((1u << lane) - 1u));
       const float2 xy = prefilter_src_xy(T * e.x + B * e.y + n * e.z, W0, H0);
-      const int iy = min(max((int)floorf(xy.y), 0), H0 - 1);
+      const int iy = min(max((int)floorf(xy.y), -1), H0 - 1) + 1;
       s_key[q] = ((unsigned)iy << 16) | (unsigned)q;
     }
   }
   int P = 1;
   while (P < ns) P <<= 1;
-  for (int q = ns + tid; q < P; q += kPrefilterThreads) s_key[q] = 0xffffffffu;
+  for (int q = ns + tid; q < P; q += THREADS) s_key[q] = 0xffffffffu;
   __syncthreads();
   for (int k = 2; k <= P; k <<= 1) {
     for (int jj = k >> 1; jj > 0; jj >>= 1) {
-      for (int q = tid; q < P; q += kPrefilterThreads) {
+      for (int q = tid; q < P; q += THREADS) {
         const int o = q ^ jj;
         if (o > q) {
           const unsigned a = s_key[q], b = s_key[o];
@@ -438,37 +431,65 @@ __global__ void __launch_bounds__(kPrefilterThreads) k_prefilter(MapDev src, Cha
       __syncthreads();
     }
   }
-  for (int q = tid; q < ns; q += kPrefilterThreads) s_pos[s_key[q] & 0xffffu] = (unsigned short)q;
+  for (int q = tid; q < ns; q += THREADS) s_pos[s_key[q] & 0xffffu] = (unsigned short)q;
+  keyed(s_key, ns);
   __syncthreads();  // the keys are dead from here: their space takes the records
-  // pass B: the records at their sorted positions; the weight sum sum_k n.l_k (the same for every
-  // texel of the level), summed in sample order
+  // pass B: the records at their sorted positions; the weights summed in sample order
   float wpart = 0.0f;
-  for (int gi = warp; gi < groups; gi += kPrefilterThreads / 32) {
+  for (int gi = warp; gi < groups; gi += THREADS / 32) {
     int sidx = gi * 32 + lane;
     float4 e = sidx < N ? prefilter_sample(sidx, a2, invN) : make_float4(0, 0, 0, 0);
     bool keep = sidx < N && e.z > 0.0f;
     unsigned bal = __ballot_sync(0xffffffffu, keep);
     if (keep) {
-      const int q = s_base[gi] + __popc(bal & ((1u << lane) - 1u));
-      const float2 xy = prefilter_src_xy(T * e.x + B * e.y + n * e.z, W0, H0);
-      const float xf = floorf(xy.x), yf = floorf(xy.y);
-      const float fx = xy.x - xf, fy = xy.y - yf;
-      const float wt = e.z * (1.0f - fy), wb = e.z * fy;
-      const int p = s_pos[q];
-      if (INT_SHIFT)
-        s_w[p] = make_float4(wt * (1.0f - fx), wt * fx, wb * (1.0f - fx), wb * fx);
-      else
-        s_w[p] = make_float4(wt, wb, xy.x, 0.0f);
-      s_xy[p] = make_int2((int)xf, (int)yf);
+      const int q = sh.base[gi] + __popc(bal & ((1u << lane) - 1u));
+      emit(s_pos[q], e, prefilter_src_xy(T * e.x + B * e.y + n * e.z, W0, H0));
       wpart += e.z;
     }
   }
   wpart = warp_sum(wpart);
-  if (lane == 0) s_wsum[warp] = wpart;
+  if (lane == 0) sh.wsum[warp] = wpart;
   __syncthreads();
-  float wsum = 0.0f;
+  wsum = 0.0f;
 #pragma unroll
-  for (int w = 0; w < kPrefilterThreads / 32; ++w) wsum += s_wsum[w];
+  for (int w = 0; w < THREADS / 32; ++w) wsum += sh.wsum[w];
+  return ns;
+}
+
+// Per kept sample, for texel 0 of the row, in order of source row: INT_SHIFT (W0 a multiple of
+// Wm) stores the four bilinear weights times n.l and (column, row); otherwise the two row weights
+// times n.l and the source x coordinate (the column fraction then varies along the row), and the
+// row.  Samples are visited in order of their source row so that consecutive samples read the
+// same two rows, which stay in L1.
+template <bool INT_SHIFT>
+__global__ void __launch_bounds__(kPrefilterThreads) k_prefilter(MapDev src, ChainDev ch, int N) {
+  extern __shared__ __align__(16) float4 s_pf[];
+  __shared__ PrefilterShared sh;
+  __shared__ float3 s_sum[kPrefilterThreads * 2];  // the shares' sums
+  griddep_launch_dependents();  // k_prefilter_rows does other levels at the same time
+  float4* s_w = s_pf;
+  int2* s_xy = (int2*)(s_pf + N);
+  unsigned short* s_pos = (unsigned short*)(s_xy + N);
+  const int m = blockIdx.y + ch.first;
+  const int W = ch.W[m], H = ch.H[m];
+  const int segs = (W + kPrefilterSeg - 1) / kPrefilterSeg;
+  const int j = blockIdx.x / segs, i0 = (blockIdx.x - j * segs) * kPrefilterSeg;
+  if (j >= H) return;  // block-uniform
+  const int W0 = src.W, H0 = src.H;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  float wsum;
+  const int ns = prefilter_records<kPrefilterThreads>(
+      sh, (unsigned*)s_pf, s_pos, m, ch.M, j, W, H, W0, H0, N, wsum, [](const unsigned*, int) {},
+      [&](int p, float4 e, float2 xy) {
+        const float xf = floorf(xy.x), yf = floorf(xy.y);
+        const float fx = xy.x - xf, fy = xy.y - yf;
+        const float wt = e.z * (1.0f - fy), wb = e.z * fy;
+        if (INT_SHIFT)
+          s_w[p] = make_float4(wt * (1.0f - fx), wt * fx, wb * (1.0f - fx), wb * fx);
+        else
+          s_w[p] = make_float4(wt, wb, xy.x, 0.0f);
+        s_xy[p] = make_int2((int)xf, (int)yf);
+      });
   const float inv = 1.0f / wsum;
   const int step_i = W0 / W;  // INT_SHIFT: whole source columns per texel
   const float step_f = (float)W0 / (float)W;
@@ -477,9 +498,11 @@ __global__ void __launch_bounds__(kPrefilterThreads) k_prefilter(MapDev src, Cha
     // g = 0..3, with the tap column d = l & 1 (columns x0 + s i + d), so a warp's loads of one
     // row and group are 32 consecutive texels at level 1 (s = 2); the two lanes of a texel add
     // their sums at the end.
+    // A segment of at most 256 texels leaves warps over: these take shares of the samples (`split`).
+    const int cols = (min(W - i0, kPrefilterSeg) + 63) / 64;  // warps side by side
+    const int across = cols > 4 ? 8 : (cols > 2 ? 4 : cols), split = warp / across, splits = 8 / across;
     const int t = lane >> 1, dl = lane & 1;
-    const int wbase = i0 + warp * 64;
-    if (wbase >= W) return;  // warp-uniform, after the last barrier
+    const int wbase = i0 + (warp - split * across) * 64;
     int col[4];
     bool ong[4];
     float3 acc[4], part[4];
@@ -490,8 +513,9 @@ __global__ void __launch_bounds__(kPrefilterThreads) k_prefilter(MapDev src, Cha
       col[g] = min(i, W - 1) * step_i + dl;
       acc[g] = part[g] = f3(0, 0, 0);
     }
+    int since = 0;
 #pragma unroll 2
-    for (int q = 0; q < ns; ++q) {
+    for (int q = split; q < (ong[0] ? ns : 0); q += splits) {
       const float4 w = s_w[q];
       const int2 xy = s_xy[q];
       const int r0 = max(xy.y, 0) * W0, r1 = min(xy.y + 1, H0 - 1) * W0;
@@ -506,7 +530,7 @@ __global__ void __launch_bounds__(kPrefilterThreads) k_prefilter(MapDev src, Cha
         part[g].y = fmaf(wa, a.y, fmaf(wb, p.y, part[g].y));
         part[g].z = fmaf(wa, a.z, fmaf(wb, p.z, part[g].z));
       }
-      if ((q & 63) == 63) {  // fold every 64 samples' plain sums into the running sums
+      if ((++since & 63) == 0) {  // fold every 64 samples' plain sums into the running sums
 #pragma unroll
         for (int g = 0; g < 4; ++g) {
           acc[g] = acc[g] + part[g];
@@ -516,30 +540,42 @@ __global__ void __launch_bounds__(kPrefilterThreads) k_prefilter(MapDev src, Cha
     }
 #pragma unroll
     for (int g = 0; g < 4; ++g) {
-      if (!ong[g]) continue;
       float3 v = acc[g] + part[g];
       v.x += __shfl_xor_sync(0xffffffffu, v.x, 1);
       v.y += __shfl_xor_sync(0xffffffffu, v.y, 1);
       v.z += __shfl_xor_sync(0xffffffffu, v.z, 1);
+      acc[g] = v;
+      if (splits > 1 && dl == 0) s_sum[warp * 64 + 16 * g + t] = v;
+    }
+    if (splits > 1) __syncthreads();  // block-uniform
+    if (split > 0) return;
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
       const int i = wbase + 16 * g + t;
-      if (dl == 0 && i < W) {
-        const float3 o = v * inv;
-        ch.dst[m][(long long)j * W + i] = make_float4(o.x, o.y, o.z, 1.0f);
-      }
+      if (dl || !ong[g] || i >= W) continue;
+      float3 v = acc[g];
+      for (int k = 1; k < splits; ++k) v = v + s_sum[(warp + k * across) * 64 + 16 * g + t];
+      const float3 o = v * inv;
+      ch.dst[m][(long long)j * W + i] = make_float4(o.x, o.y, o.z, 1.0f);
     }
     return;
   }
+  // a thread per texel, or per texel and share of the samples where the segment has at most 128
+  const int n = min(W - i0, kPrefilterSeg);
+  const int across = n > 128 ? 256 : (n > 64 ? 128 : (n > 32 ? 64 : 32)), split = tid / across;
+  const int splits = kPrefilterThreads / across, me = tid - split * across;
   int ii[kPrefilterTexels];
   bool on[kPrefilterTexels];  // block-uniform: whether the segment has a texel group c
   float3 acc[kPrefilterTexels], part[kPrefilterTexels];
 #pragma unroll
   for (int c = 0; c < kPrefilterTexels; ++c) {
-    on[c] = i0 + c * kPrefilterThreads < W;
-    ii[c] = min(i0 + c * kPrefilterThreads + tid, W - 1);  // duplicates of the last texel are not stored
+    on[c] = c * kPrefilterThreads < n;
+    ii[c] = min(i0 + c * kPrefilterThreads + me, W - 1);  // duplicates of the last texel are not stored
     acc[c] = part[c] = f3(0, 0, 0);
   }
+  int since = 0;
 #pragma unroll 2
-  for (int q = 0; q < ns; ++q) {
+  for (int q = split; q < ns; q += splits) {
     const float4 w = s_w[q];
     const int2 xy = s_xy[q];
     const int r0 = max(xy.y, 0) * W0, r1 = min(xy.y + 1, H0 - 1) * W0;
@@ -558,7 +594,7 @@ __global__ void __launch_bounds__(kPrefilterThreads) k_prefilter(MapDev src, Cha
       part[c].y = fmaf(wq.x, a.y, fmaf(wq.y, b.y, fmaf(wq.z, p.y, fmaf(wq.w, d.y, part[c].y))));
       part[c].z = fmaf(wq.x, a.z, fmaf(wq.y, b.z, fmaf(wq.z, p.z, fmaf(wq.w, d.z, part[c].z))));
     }
-    if ((q & 63) == 63) {  // fold every 64 samples' plain sums into the running sums
+    if ((++since & 63) == 0) {  // fold every 64 samples' plain sums into the running sums
 #pragma unroll
       for (int c = 0; c < kPrefilterTexels; ++c) {
         acc[c] = acc[c] + part[c];
@@ -566,14 +602,213 @@ __global__ void __launch_bounds__(kPrefilterThreads) k_prefilter(MapDev src, Cha
       }
     }
   }
+  if (splits > 1) {  // block-uniform
+    s_sum[tid] = acc[0] + part[0];
+    __syncthreads();
+    if (split > 0) return;
+  }
 #pragma unroll
   for (int c = 0; c < kPrefilterTexels; ++c) {
-    const int i = i0 + c * kPrefilterThreads + tid;
+    const int i = i0 + c * kPrefilterThreads + me;
     if (on[c] && i < W) {
-      const float3 o = (acc[c] + part[c]) * inv;
+      float3 v = acc[c] + part[c];
+      for (int k = 1; k < splits; ++k) v = v + s_sum[me + k * across];
+      const float3 o = v * inv;
       ch.dst[m][(long long)j * W + i] = make_float4(o.x, o.y, o.z, 1.0f);
     }
   }
+}
+
+// Levels whose texels are a power of two of source columns apart: the block of a row stages every
+// source row its samples touch, once, in shared memory as three channel planes of phases
+// (column c = phase + phases * k at [phase][k]), so that a tap of all texels of the row is three
+// conflict-free reads of consecutive words, 12 bytes per texel instead of the 16 of an L1 read whose
+// lines are half, a quarter, ... used.  A thread owns two neighbouring texels (their columns are
+// `step` apart, so a row is staged in 2 step phases and one index serves all four taps); threads left
+// over take shares of the samples.  Bound by shared-memory bandwidth (two rows x two columns x 12
+// bytes per texel and sample; ncu: 78% of the LSU data pipe): levels 1 .. 7 of a 2048 x 1024
+// environment at 1024 samples 2545 us with every level read through L1, 2060 us with levels 1 and 2
+// here and the others, whose spare warps now share the samples, beside them.
+constexpr int kRowsThreads = 512, kRowsMaxW = 2048, kRowsMaxH = 2048;
+constexpr int kRowsMinW = 128;  // texels per row of a level
+// Above a step of 4 a source row is staged for too few texels: the lighting set of a 2048 x 1024
+// environment takes 2316, 2145 and 2248 us with steps up to 2, 4 and 8.
+constexpr int kRowsMaxStep = 4;
+constexpr int kRowsPlane = kRowsMaxW + 32;     // words per channel: phases padded by 32 / phases words
+constexpr int kRowsSlot = 3 * kRowsPlane;      // words per staged row; three of them: two in use, one being filled
+
+// A sample as the taps read it: byte offset of k for texel 0, then byte offsets of the phases of the
+// two tap columns of an even texel and of the odd texel after it (relative to k, so 4 more where a
+// column belongs to the next k).
+struct RowsTap {
+  unsigned k;
+  unsigned even, odd;  // first column | second column << 16
+  unsigned pad;
+};
+
+__device__ __forceinline__ RowsTap rows_tap(int c, int step, int phases, int phase_words) {
+  const int p = c & (phases - 1);
+  auto at = [&](int d) { return (unsigned)(((p + d) & (phases - 1)) * phase_words + (p + d >= phases ? 1 : 0)) * 4u; };
+  return RowsTap{(unsigned)(c / phases) * 4u, at(0) | (at(1) << 16), at(step) | (at(step + 1) << 16), 0u};
+}
+
+extern __shared__ __align__(16) float s_rows[];
+
+// Adds samples from, from + stride, ... below to, between the rows in slots SLOT and SLOT + 1 (modulo
+// 3), to the texel pair whose even texel is k4 / 4 pairs along the row of n4 / 4 pairs.
+template <int SLOT>
+__device__ __forceinline__ void prefilter_taps(float3 (&part)[2], const float4* s_w, const RowsTap* s_tap, int from,
+                                               int to, int stride, unsigned k4, unsigned n4) {
+  constexpr int kTop = SLOT * kRowsSlot, kBot = (SLOT + 1) % 3 * kRowsSlot;
+  for (int q = from; q < to; q += stride) {
+    const float4 w = s_w[q];
+    const uint4 t = *(const uint4*)(s_tap + q);
+    unsigned k = t.x + k4;
+    k = min(k, k - n4);  // wrapped round the row
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+      const unsigned o = g ? t.z : t.y;
+      const float* a = (const float*)((const char*)s_rows + (k + (o & 0xffffu)));
+      const float* b = (const float*)((const char*)s_rows + (k + (o >> 16)));
+      part[g].x = fmaf(w.x, a[kTop], fmaf(w.y, b[kTop], fmaf(w.z, a[kBot], fmaf(w.w, b[kBot], part[g].x))));
+      part[g].y = fmaf(w.x, a[kTop + kRowsPlane], fmaf(w.y, b[kTop + kRowsPlane],
+                  fmaf(w.z, a[kBot + kRowsPlane], fmaf(w.w, b[kBot + kRowsPlane], part[g].y))));
+      part[g].z = fmaf(w.x, a[kTop + 2 * kRowsPlane], fmaf(w.y, b[kTop + 2 * kRowsPlane],
+                  fmaf(w.z, a[kBot + 2 * kRowsPlane], fmaf(w.w, b[kBot + 2 * kRowsPlane], part[g].z))));
+    }
+  }
+}
+
+// s_list: the `rows` source rows that are read (r + 1, -1 and H0 the clamped edges), in ascending
+// order, a sample's two rows next to each other.
+__device__ __forceinline__ void prefilter_row(const float4* s_w, const RowsTap* s_tap, const unsigned short* s_start,
+                                              const unsigned short* s_list, int rows, const MapDev& src,
+                                              float4* __restrict__ dst, int W, int phases, int phase_words, float inv) {
+  const int tid = threadIdx.x, W0 = src.W, H0 = src.H;
+  const int pairs = W / 2, share = tid / pairs, shares = kRowsThreads / pairs, me = tid - share * pairs;
+  constexpr int kLoads = kRowsMaxW / kRowsThreads;
+  float4 v[kLoads];
+  auto load = [&](int k0) {
+    const float4* row = src.texels + (size_t)min(max((int)s_list[k0] - 1, 0), H0 - 1) * W0;
+#pragma unroll
+    for (int k = 0; k < kLoads; ++k)
+      if (tid + k * kRowsThreads < W0) v[k] = __ldg(row + tid + k * kRowsThreads);
+  };
+  const int log2p = 31 - __clz(phases);
+  auto store = [&](int slot) {
+#pragma unroll
+    for (int k = 0; k < kLoads; ++k) {
+      const int c = tid + k * kRowsThreads;
+      if (c >= W0) continue;
+      float* q = s_rows + slot * kRowsSlot + (c & (phases - 1)) * phase_words + (c >> log2p);
+      q[0] = v[k].x, q[kRowsPlane] = v[k].y, q[2 * kRowsPlane] = v[k].z;
+      if (c < phases) {  // each phase's first column once more after its last
+        q += pairs;
+        q[0] = v[k].x, q[kRowsPlane] = v[k].y, q[2 * kRowsPlane] = v[k].z;
+      }
+    }
+  };
+  float3 acc[2], part[2];
+  acc[0] = acc[1] = part[0] = part[1] = f3(0, 0, 0);
+  load(0);
+  store(0);
+  load(1);
+  store(1);
+  __syncthreads();
+  int since = 0;
+  for (int k = 0, slot = 0; k + 1 < rows; ++k) {
+    if (k + 2 < rows) load(k + 2);
+    const int from = s_start[s_list[k]], to = s_start[s_list[k] + 1];  // the samples between rows k and k + 1
+    if (share < shares) {
+      if (slot == 0) prefilter_taps<0>(part, s_w, s_tap, from + share, to, shares, 4u * me, 4u * pairs);
+      if (slot == 1) prefilter_taps<1>(part, s_w, s_tap, from + share, to, shares, 4u * me, 4u * pairs);
+      if (slot == 2) prefilter_taps<2>(part, s_w, s_tap, from + share, to, shares, 4u * me, 4u * pairs);
+    }
+    since += to - from;
+    if (since >= 64) {  // fold the plain sums into the running sums
+      since = 0;
+#pragma unroll
+      for (int g = 0; g < 2; ++g) {
+        acc[g] = acc[g] + part[g];
+        part[g] = f3(0, 0, 0);
+      }
+    }
+    if (k + 2 < rows) store(slot == 0 ? 2 : slot - 1);  // the slot of row k - 1
+    slot = slot == 2 ? 0 : slot + 1;
+    __syncthreads();
+  }
+  float3 sum[2] = {acc[0] + part[0], acc[1] + part[1]};
+  if (shares > 1) {  // block-uniform; the staged rows are dead
+    float3* s_sum = (float3*)s_rows;
+    s_sum[2 * tid] = sum[0];
+    s_sum[2 * tid + 1] = sum[1];
+    __syncthreads();
+    if (share == 0)
+      for (int k = 1; k < shares; ++k) {
+        sum[0] = sum[0] + s_sum[2 * (tid + k * pairs)];
+        sum[1] = sum[1] + s_sum[2 * (tid + k * pairs) + 1];
+      }
+  }
+  if (share > 0) return;
+#pragma unroll
+  for (int g = 0; g < 2; ++g) {
+    const float3 o = sum[g] * inv;
+    dst[2 * me + g] = make_float4(o.x, o.y, o.z, 1.0f);
+  }
+}
+
+// Dynamic shared memory: the staged rows, N float4 weights (first the sort keys), N taps, N sorted
+// positions, H0 + 3 first samples (of source row r at [r + 1]), the list of source rows.
+size_t rows_shared_bytes(int N, int H0) {
+  return 4 * (size_t)(3 * kRowsSlot) + (sizeof(float4) + sizeof(RowsTap) + 2) * (size_t)N + 4 * (size_t)(H0 + 3);
+}
+
+__global__ void __launch_bounds__(kRowsThreads, 2) k_prefilter_rows(MapDev src, ChainDev ch, int N) {
+  __shared__ PrefilterShared rec;
+  __shared__ int s_rows_n;
+  const int m = blockIdx.y + ch.first, j = blockIdx.x, W = ch.W[m], H = ch.H[m], H0 = src.H, W0 = src.W;
+  if (j < H) {  // block-uniform
+    float4* s_w = (float4*)(s_rows + 3 * kRowsSlot);
+    RowsTap* s_tap = (RowsTap*)(s_w + N);
+    unsigned short* s_pos = (unsigned short*)(s_tap + N);
+    unsigned short* s_start = s_pos + N;
+    unsigned short* s_list = s_start + H0 + 3;
+    const int step = 1 << m, phases = 2 * step, phase_words = (W0 + 32) / phases;
+    float wsum;
+    prefilter_records<kRowsThreads>(
+        rec, (unsigned*)s_w, s_pos, m, ch.M, j, W, H, W0, H0, N, wsum,
+        [&](const unsigned* key, int n) {
+          // start[k] = number of samples whose source row + 1 is below k
+          for (int q = threadIdx.x; q <= n; q += kRowsThreads) {
+            const int lo = q > 0 ? (int)(key[q - 1] >> 16) + 1 : 0, hi = q < n ? (int)(key[q] >> 16) : H0 + 2;
+            for (int k = lo; k <= hi; ++k) s_start[k] = (unsigned short)q;
+          }
+        },
+        [&](int p, float4 e, float2 xy) {
+          const float xf = floorf(xy.x), yf = floorf(xy.y);
+          const float fx = xy.x - xf, fy = xy.y - yf;
+          const float wt = e.z * (1.0f - fy), wb = e.z * fy;
+          s_w[p] = make_float4(wt * (1.0f - fx), wt * fx, wb * (1.0f - fx), wb * fx);
+          const int c = (int)xf;
+          s_tap[p] = rows_tap(c < 0 ? c + W0 : (c >= W0 ? c - W0 : c), step, phases, phase_words);
+        });
+    // the source rows with a sample (between them and the next) and the rows after these
+    if (threadIdx.x < 32) {
+      int n = 0;
+      for (int r0 = 0; r0 < H0 + 2; r0 += 32) {
+        const int r = r0 + threadIdx.x;  // source row + 1
+        const bool need = r < H0 + 2 && s_start[r + 1] > s_start[max(r - 1, 0)];
+        const unsigned bal = __ballot_sync(0xffffffffu, need);
+        if (need) s_list[n + __popc(bal & ((1u << threadIdx.x) - 1u))] = (unsigned short)r;
+        n += __popc(bal);
+      }
+      if (threadIdx.x == 0) s_rows_n = n;
+    }
+    __syncthreads();
+    float4* dst = ch.dst[m] + (long long)j * W;
+    prefilter_row(s_w, s_tap, s_start, s_list, s_rows_n, src, dst, W, phases, phase_words, 1.0f / wsum);
+  }
+  griddep_wait();  // launched beside k_prefilter: complete only after it
 }
 
 static epbr_status validate_ibl_for(const epbr_ibl* ibl, int We, int He) {
@@ -761,33 +996,51 @@ extern "C" epbr_status epbr_prefilter(const epbr_env* env, int32_t N, const epbr
   if (ibl->num_levels < 2) return ok();
   ChainDev ch;
   ch.M = ibl->num_levels;
-  ch.nlev = ibl->num_levels - 1;
-  ch.off[0] = 0;
   for (int m = 0; m < EPBR_MAX_LEVELS; ++m) {
     ch.W[m] = ibl->level_width[m];
     ch.H[m] = ibl->level_height[m];
     ch.dst[m] = (float4*)ibl->level[m];
   }
-  for (int li = 0; li < ch.nlev; ++li) ch.off[li + 1] = ch.off[li] + (long long)ch.W[li + 1] * ch.H[li + 1];
-  MapDev src{(const float4*)env->texels, env->width, env->height};
-  // one block per row of every level (level 1 has the most rows); whole-column shifts when every
-  // level's width divides the source width
-  bool int_shift = true;
-  for (int m = 1; m < ibl->num_levels; ++m) int_shift = int_shift && env->width % ch.W[m] == 0;
-  unsigned most = 0;
-  for (int m = 1; m < ibl->num_levels; ++m)
-    most = std::max(most, (unsigned)(ch.H[m] * ((ch.W[m] + kPrefilterSeg - 1) / kPrefilterSeg)));
-  dim3 grid(most, (unsigned)ch.nlev);
-  const size_t smem = (size_t)N * (sizeof(float4) + sizeof(int2) + sizeof(unsigned short));
-  void (*k)(MapDev, ChainDev, int) = int_shift ? k_prefilter<true> : k_prefilter<false>;
-  if (smem > 48 * 1024 &&
-      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return fail(EPBR_ERR_CUDA, "prefilter: shared-memory attribute: %s", cudaGetErrorString(cudaGetLastError()));
-  // a small shared-memory carve-out leaves most of the SM's 256 KB to L1, which holds the source
-  // rows the resident blocks read (two rows of up to 16 KB per block)
-  cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 50);  // a hint; failure is harmless
-  k<<<grid, kPrefilterThreads, smem, s>>>(src, ch, N);
-  if ((st = check_launch("k_prefilter"))) return st;
+  const int W0 = env->width, H0 = env->height;
+  MapDev src{(const float4*)env->texels, W0, H0};
+  // levels 1 .. rows by k_prefilter_rows: texels 2 or 4 source columns apart, texel pairs of whole warps
+  int rows = 0;
+  while (rows + 1 < ch.M && (2 << rows) <= kRowsMaxStep && W0 <= kRowsMaxW && H0 <= kRowsMaxH &&
+         W0 % (64 * (2 << rows)) == 0 && W0 / (2 << rows) >= kRowsMinW)
+    ++rows;
+  // the others one block per row (level rows + 1 has the most rows), before it: the two run side
+  // by side; whole-column shifts when every level's width divides the source width
+  ch.first = rows + 1;
+  if (ch.first < ch.M) {
+    bool int_shift = true;
+    for (int m = ch.first; m < ch.M; ++m) int_shift = int_shift && W0 % ch.W[m] == 0;
+    unsigned most = 0;
+    for (int m = ch.first; m < ch.M; ++m)
+      most = std::max(most, (unsigned)(ch.H[m] * ((ch.W[m] + kPrefilterSeg - 1) / kPrefilterSeg)));
+    const size_t smem = (size_t)N * (sizeof(float4) + sizeof(int2) + sizeof(unsigned short));
+    void (*k)(MapDev, ChainDev, int) = int_shift ? k_prefilter<true> : k_prefilter<false>;
+    if (smem > 48 * 1024 &&
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+      return fail(EPBR_ERR_CUDA, "prefilter: shared-memory attribute: %s", cudaGetErrorString(cudaGetLastError()));
+    // a small shared-memory carve-out leaves most of the SM's 256 KB to L1, which holds the source
+    // rows the resident blocks read (two rows of up to 16 KB per block)
+    cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 50);  // a hint; failure is harmless
+    k<<<dim3(most, (unsigned)(ch.M - ch.first)), kPrefilterThreads, smem, s>>>(src, ch, N);
+    if ((st = check_launch("k_prefilter"))) return st;
+  }
+  if (rows > 0) {
+    const bool early = ch.first < ch.M;
+    ch.first = 1;
+    const size_t smem = rows_shared_bytes(N, H0);
+    if (cudaFuncSetAttribute(k_prefilter_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+      return fail(EPBR_ERR_CUDA, "prefilter: shared-memory attribute: %s", cudaGetErrorString(cudaGetLastError()));
+    cudaError_t e = launch_kernel(k_prefilter_rows, dim3(ch.H[1], rows), dim3(kRowsThreads), smem, s, early, src, ch, N);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      return fail(EPBR_ERR_CUDA, "k_prefilter_rows: %s", cudaGetErrorString(e));
+    }
+    if ((st = check_launch("k_prefilter_rows"))) return st;
+  }
   return ok();
 }
 
