@@ -6,12 +6,15 @@
 //                      clamp to the edge never reaches outside the block, because tiles are
 //                      aligned to powers of two.  The full-resolution bright map is never stored.
 //   k_bloom_blur       every level in one launch: a 32x16 texel tile plus an R-texel halo in shared
-//                      memory, rows then columns of the separable Gaussian
+//                      memory, rows then columns of the separable Gaussian, several outputs per
+//                      thread from one window of registers
 //   k_bloom_composite  one 2x2 pixel quad per thread: X + s * sum_k bilinear(level k at the pixel
 //                      centre), HDR store and / or the fused tone map.  On level 1 the quad's four
 //                      bilinear footprints lie in a 3x3 texel block; on level k >= 2 both pixels of
 //                      a row (or column) pair fall in the same texel cell, so the quad loads 2x2
 //                      texels per level.  Each pixel's arithmetic is the per-pixel bilinear.
+// The blur and the composite are launched as programmatic dependents (they wait before they read or
+// write anything of the kernels before them, except for the composite's reads of the input image).
 #include <string.h>
 
 #include <cmath>
@@ -49,6 +52,7 @@ __global__ void __launch_bounds__(kBloomTX* kBloomTY)
     k_bloom_pyramid(const void* __restrict__ hdr, long long pitch, int W, int H, float threshold, BloomDev d) {
   __shared__ float4 s_a[32 * 32];  // levels 1, 3, 5 of the block's tile
   __shared__ float4 s_b[16 * 16];  // levels 2, 4
+  griddep_launch_dependents();
   const int tid = threadIdx.y * kBloomTX + threadIdx.x;
   {
     const BloomLevel& l1 = d.lev[1];
@@ -111,71 +115,85 @@ __global__ void __launch_bounds__(kBloomTX* kBloomTY)
   }
 }
 
-__global__ void __launch_bounds__(kBloomTX* kBloomTY) k_bloom_blur(BloomDev d) {
-  constexpr int TW = kBlurTW + 2 * kBloomMaxR, TH = kBlurTH + 2 * kBloomMaxR;
+// A texel's four channels as two FP32x2 pairs.
+struct Pair4 {
+  float2 a, b;
+};
+__device__ __forceinline__ Pair4 pair4(float4 v) { return Pair4{make_float2(v.x, v.y), make_float2(v.z, v.w)}; }
+__device__ __forceinline__ Pair4 pair_fma(float t, Pair4 v, Pair4 c) {  // t v + c
+  return Pair4{pfma(dup2(t), v.a, c.a), pfma(dup2(t), v.b, c.b)};
+}
+
+// Each output's sum runs over its taps in ascending order.  A thread's window of 4 + 2R (rows) or 2 +
+// 2R (columns) texels serves its 4 or 2 outputs, 3 + 1/2 + 5 shared-memory reads of 16 bytes per
+// output at R = 4 (with the halo) instead of 22.  Bound by latency in the short launch.
+template <int R>
+__global__ void __launch_bounds__(kBloomTX* kBloomTY) k_bloom_blur(const __grid_constant__ BloomDev d) {
+  // an odd row of 16-byte texels: eight lanes one row apart read eight different bank groups
+  constexpr int TW = (kBlurTW + 2 * R) | 1, TH = kBlurTH + 2 * R, kTaps = 2 * R + 1;
   __shared__ float4 s_in[TH][TW];
-  __shared__ float4 s_row[TH][kBlurTW];
-  __shared__ float s_w[2 * kBloomMaxR + 1];
+  __shared__ float4 s_row[TH][kBlurTW + 1];
+  griddep_wait();  // launched early: the pyramid is complete
+  griddep_launch_dependents();
   const int tid = threadIdx.y * kBloomTX + threadIdx.x;
-  const int R = d.R;
-  if (tid <= 2 * R) s_w[tid] = d.w[tid];
   int b = blockIdx.x, k = 1;
 #pragma unroll
   for (int q = 2; q < kBloomMaxLevels; ++q)
     if (q < d.L && b >= d.tile_start[q]) k = q;
-  BloomLevel lv = d.lev[1];
-  int tiles_x = d.tiles_x[1];
-#pragma unroll
-  for (int q = 2; q < kBloomMaxLevels; ++q)
-    if (q == k) lv = d.lev[q], tiles_x = d.tiles_x[q];
+  const BloomLevel lv = d.lev[k];
+  const int tiles_x = d.tiles_x[k];
   b -= d.tile_start[k];
   const int by = b / tiles_x;
   const int x0 = (b - by * tiles_x) * kBlurTW, y0 = by * kBlurTH;
-  const int tw = kBlurTW + 2 * R, th = kBlurTH + 2 * R;
-  for (int ty = threadIdx.y; ty < th; ty += kBloomTY) {
+  for (int ty = threadIdx.y; ty < TH; ty += kBloomTY) {
     const float4* row = lv.pyr + (size_t)min(max(y0 - R + ty, 0), lv.H - 1) * lv.W;
-    for (int tx = threadIdx.x; tx < tw; tx += kBloomTX) s_in[ty][tx] = __ldg(row + min(max(x0 - R + tx, 0), lv.W - 1));
+    for (int tx = threadIdx.x; tx < kBlurTW + 2 * R; tx += kBloomTX) s_in[ty][tx] = row[min(max(x0 - R + tx, 0), lv.W - 1)];
   }
   __syncthreads();
-  for (int ty = threadIdx.y; ty < th; ty += kBloomTY) {
-    float3 sum = f3(0, 0, 0);
+  // rows: four neighbouring outputs per thread, lanes down the rows
+  for (int q = tid; q < TH * (kBlurTW / 4); q += kBloomTX * kBloomTY) {
+    const int g = q / TH, ty = q - g * TH;
+    Pair4 v[4 + 2 * R];
 #pragma unroll
-    for (int t = 0; t <= 2 * kBloomMaxR; ++t) {
-      if (t > 2 * R) break;
-      sum = sum + s_w[t] * xyz(s_in[ty][threadIdx.x + t]);
+    for (int t = 0; t < 4 + 2 * R; ++t) v[t] = pair4(s_in[ty][4 * g + t]);
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+      Pair4 sum = {make_float2(0, 0), make_float2(0, 0)};
+#pragma unroll
+      for (int t = 0; t < kTaps; ++t) sum = pair_fma(d.w[t], v[o + t], sum);
+      s_row[ty][4 * g + o] = make_float4(sum.a.x, sum.a.y, sum.b.x, 0.0f);
     }
-    s_row[ty][threadIdx.x] = make_float4(sum.x, sum.y, sum.z, 0.0f);
   }
   __syncthreads();
-  const int x = x0 + threadIdx.x;
+  // columns: two neighbouring outputs per thread
+  const int x = x0 + threadIdx.x, ly = 2 * threadIdx.y;
+  Pair4 v[2 + 2 * R];
 #pragma unroll
-  for (int r = 0; r < kBlurTH / kBloomTY; ++r) {
-    const int ly = threadIdx.y + r * kBloomTY, y = y0 + ly;
-    if (x >= lv.W || y >= lv.H) continue;
-    float3 sum = f3(0, 0, 0);
+  for (int t = 0; t < 2 + 2 * R; ++t) v[t] = pair4(s_row[ly + t][threadIdx.x]);
 #pragma unroll
-    for (int t = 0; t <= 2 * kBloomMaxR; ++t) {
-      if (t > 2 * R) break;
-      sum = sum + s_w[t] * xyz(s_row[ly + t][threadIdx.x]);
-    }
-    lv.blr[(size_t)y * lv.W + x] = make_float4(sum.x, sum.y, sum.z, 0.0f);
+  for (int o = 0; o < 2; ++o) {
+    const int y = y0 + ly + o;
+    Pair4 sum = {make_float2(0, 0), make_float2(0, 0)};
+#pragma unroll
+    for (int t = 0; t < kTaps; ++t) sum = pair_fma(d.w[t], v[o + t], sum);
+    if (x < lv.W && y < lv.H) lv.blr[(size_t)y * lv.W + x] = make_float4(sum.a.x, sum.a.y, sum.b.x, 0.0f);
   }
 }
 
-__device__ __forceinline__ float3 lerp3(float3 a, float3 b, float t) { return a + t * (b - a); }
-
-// The bilinear value at fractions (fx, fy) of the texel cell with corners a (top left), b (top
-// right), p (bottom left), q (bottom right).
-__device__ __forceinline__ float3 bilerp(float3 a, float3 b, float3 p, float3 q, float fx, float fy) {
-  float3 top = lerp3(a, b, fx), bot = lerp3(p, q, fx);
-  return lerp3(top, bot, fy);
+// a + t (b - a)
+__device__ __forceinline__ Pair4 pair_lerp(Pair4 a, Pair4 b, float t) {
+  const float2 na = make_float2(-a.a.x, -a.a.y), nb = make_float2(-a.b.x, -a.b.y);
+  return Pair4{pfma(dup2(t), padd(b.a, na), a.a), pfma(dup2(t), padd(b.b, nb), a.b)};
 }
 
 // Adds s * sum_k (level k sampled bilinearly at the pixel centre) to the quad's four pixels
 // c[b][a] = pixel (2 qi + a, 2 qj + b).  Pixel x lies at texel coordinate u = (x + 1/2) 2^-k - 1/2
-// of level k, exact in FP32 for the admitted sizes.
+// of level k, exact in FP32 for the admitted sizes.  The channels are processed in packed FP32x2
+// pairs, which lie in the registers as the texels are loaded.
 __device__ __forceinline__ void bloom_add_quad(const BloomDev& d, float strength, int qi, int qj, float3 (&c)[2][2]) {
-  float3 add[2][2] = {{f3(0, 0, 0), f3(0, 0, 0)}, {f3(0, 0, 0), f3(0, 0, 0)}};
+  const Pair4 zero = {make_float2(0, 0), make_float2(0, 0)};
+  Pair4 add[2][2] = {{zero, zero}, {zero, zero}};
+  auto sum = [](Pair4& a, Pair4 v) { a.a = padd(a.a, v.a), a.b = padd(a.b, v.b); };
   {
     // level 1: pixel 2 qi sits at u = qi - 1/4 (cell qi-1, fraction 3/4), pixel 2 qi + 1 at
     // qi + 1/4 (cell qi, fraction 1/4): the footprints span texels qi-1 .. qi+1
@@ -186,19 +204,18 @@ __device__ __forceinline__ void bloom_add_quad(const BloomDev& d, float strength
       ci[t] = min(max(qi - 1 + t, 0), lv.W - 1);
       cj[t] = min(max(qj - 1 + t, 0), lv.H - 1);
     }
-    float3 T[3][3];
+    Pair4 row[3][2];  // each texel row at the two pixels' columns
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
-      const float4* row = lv.blr + (size_t)cj[r] * lv.W;
-#pragma unroll
-      for (int t = 0; t < 3; ++t) T[r][t] = xyz(__ldg(row + ci[t]));
+      const float4* p = lv.blr + (size_t)cj[r] * lv.W;
+      const Pair4 t0 = pair4(p[ci[0]]), t1 = pair4(p[ci[1]]), t2 = pair4(p[ci[2]]);
+      row[r][0] = pair_lerp(t0, t1, 0.75f);
+      row[r][1] = pair_lerp(t1, t2, 0.25f);
     }
 #pragma unroll
     for (int b = 0; b < 2; ++b)
 #pragma unroll
-      for (int a = 0; a < 2; ++a)
-        add[b][a] = add[b][a] + bilerp(T[b][a], T[b][a + 1], T[b + 1][a], T[b + 1][a + 1], a ? 0.25f : 0.75f,
-                                       b ? 0.25f : 0.75f);
+      for (int a = 0; a < 2; ++a) sum(add[b][a], pair_lerp(row[b][a], row[b + 1][a], b ? 0.25f : 0.75f));
   }
 #pragma unroll
   for (int k = 2; k < kBloomMaxLevels; ++k) {
@@ -219,29 +236,33 @@ __device__ __forceinline__ void bloom_add_quad(const BloomDev& d, float strength
     const int j0 = min(max(iv, 0), lv.H - 1), j1 = min(max(iv + 1, 0), lv.H - 1);
     const float4* r0 = lv.blr + (size_t)j0 * lv.W;
     const float4* r1 = lv.blr + (size_t)j1 * lv.W;
-    float3 A = xyz(__ldg(r0 + i0)), B = xyz(__ldg(r0 + i1)), P = xyz(__ldg(r1 + i0)), Q = xyz(__ldg(r1 + i1));
+    const Pair4 A = pair4(r0[i0]), B = pair4(r0[i1]), P = pair4(r1[i0]), Q = pair4(r1[i1]);
 #pragma unroll
-    for (int b = 0; b < 2; ++b)
+    for (int a = 0; a < 2; ++a) {
+      const Pair4 top = pair_lerp(A, B, u[a] - fu), bot = pair_lerp(P, Q, u[a] - fu);
 #pragma unroll
-      for (int a = 0; a < 2; ++a) add[b][a] = add[b][a] + bilerp(A, B, P, Q, u[a] - fu, v[b] - fv);
+      for (int b = 0; b < 2; ++b) sum(add[b][a], pair_lerp(top, bot, v[b] - fv));
+    }
   }
 #pragma unroll
   for (int b = 0; b < 2; ++b)
 #pragma unroll
-    for (int a = 0; a < 2; ++a) c[b][a] = c[b][a] + strength * add[b][a];
+    for (int a = 0; a < 2; ++a)
+      c[b][a] = c[b][a] + strength * f3(add[b][a].a.x, add[b][a].a.y, add[b][a].b.x);
 }
 
 template <int HF, int OF, bool LDR>
 __global__ void __launch_bounds__(kBloomTX* kBloomTY)
-    k_bloom_composite(const void* __restrict__ hdr, long long pitch, int W, int H, BloomDev d, float strength,
+    k_bloom_composite(const void* hdr, long long pitch, int W, int H, const __grid_constant__ BloomDev d, float strength,
                       void* out, long long out_pitch, float exposure, int op, uint8_t* ldr, long long ldr_pitch) {
   const int qi = blockIdx.x * kBloomTX + threadIdx.x, qj = blockIdx.y * kBloomTY + threadIdx.y;
-  if (2 * qi >= W || 2 * qj >= H) return;
+  if (2 * qi >= W || 2 * qj >= H) return;  // (a block that exits need not wait)
   float3 c[2][2];
 #pragma unroll
   for (int b = 0; b < 2; ++b)
 #pragma unroll
     for (int a = 0; a < 2; ++a) c[b][a] = load_hdr<HF>(hdr, pitch, min(2 * qi + a, W - 1), min(2 * qj + b, H - 1));
+  griddep_wait();  // launched early: only the input image is read before
   bloom_add_quad(d, strength, qi, qj, c);
 #pragma unroll
   for (int b = 0; b < 2; ++b)
@@ -292,13 +313,18 @@ extern "C" epbr_status epbr_bloom_workspace_size(int32_t width, int32_t height, 
 }
 
 template <int HF, int OF>
-static void launch_composite(dim3 g, dim3 b, cudaStream_t s, const void* hdr, long long hp, int W, int H,
-                             const BloomDev& d, float strength, void* out, long long op_, float exposure, int op,
-                             uint8_t* ldr, long long lp) {
-  if (ldr)
-    k_bloom_composite<HF, OF, true><<<g, b, 0, s>>>(hdr, hp, W, H, d, strength, out, op_, exposure, op, ldr, lp);
-  else
-    k_bloom_composite<HF, OF, false><<<g, b, 0, s>>>(hdr, hp, W, H, d, strength, out, op_, exposure, op, ldr, lp);
+static cudaError_t launch_composite(dim3 g, dim3 b, cudaStream_t s, const void* hdr, long long hp, int W, int H,
+                                    const BloomDev& d, float strength, void* out, long long op_, float exposure, int op,
+                                    uint8_t* ldr, long long lp) {
+  return launch_kernel(ldr ? k_bloom_composite<HF, OF, true> : k_bloom_composite<HF, OF, false>, g, b, 0, s, true, hdr, hp,
+                       W, H, d, strength, out, op_, exposure, op, ldr, lp);
+}
+
+static cudaError_t launch_blur(int tiles, dim3 blk, cudaStream_t s, const BloomDev& d) {
+  void (*const k[kBloomMaxR + 1])(const BloomDev) = {k_bloom_blur<0>, k_bloom_blur<1>, k_bloom_blur<2>,
+                                                     k_bloom_blur<3>, k_bloom_blur<4>, k_bloom_blur<5>,
+                                                     k_bloom_blur<6>, k_bloom_blur<7>, k_bloom_blur<8>};
+  return launch_kernel(k[d.R], dim3(tiles), blk, 0, s, true, d);
 }
 
 extern "C" epbr_status epbr_bloom(const void* hdr, int32_t hdr_format, int64_t hdr_pitch, int32_t width,
@@ -358,23 +384,23 @@ extern "C" epbr_status epbr_bloom(const void* hdr, int32_t hdr_format, int64_t h
     k_bloom_pyramid<EPBR_HDR_RGBA32F><<<gp, blk, 0, s>>>(hdr, hdr_pitch, width, height, params->threshold, d);
   else
     k_bloom_pyramid<EPBR_HDR_RGBA16F><<<gp, blk, 0, s>>>(hdr, hdr_pitch, width, height, params->threshold, d);
-  k_bloom_blur<<<tiles, blk, 0, s>>>(d);
+  cudaError_t e = launch_blur(tiles, blk, s, d);
   float exposure = tonemap ? tonemap->exposure : 1.0f;
   int op = tonemap ? tonemap->op : 0;
   dim3 g = grid_of((width + 1) / 2, (height + 1) / 2);  // one thread per 2x2 pixel quad
   bool in32 = hdr_format == EPBR_HDR_RGBA32F, out32 = !out_hdr || out_format == EPBR_HDR_RGBA32F;
-  if (in32 && out32)
-    launch_composite<EPBR_HDR_RGBA32F, EPBR_HDR_RGBA32F>(g, blk, s, hdr, hdr_pitch, width, height, d, params->strength,
-                                                         out_hdr, out_pitch, exposure, op, ldr, ldr_pitch);
-  else if (in32)
-    launch_composite<EPBR_HDR_RGBA32F, EPBR_HDR_RGBA16F>(g, blk, s, hdr, hdr_pitch, width, height, d, params->strength,
-                                                         out_hdr, out_pitch, exposure, op, ldr, ldr_pitch);
-  else if (out32)
-    launch_composite<EPBR_HDR_RGBA16F, EPBR_HDR_RGBA32F>(g, blk, s, hdr, hdr_pitch, width, height, d, params->strength,
-                                                         out_hdr, out_pitch, exposure, op, ldr, ldr_pitch);
-  else
-    launch_composite<EPBR_HDR_RGBA16F, EPBR_HDR_RGBA16F>(g, blk, s, hdr, hdr_pitch, width, height, d, params->strength,
-                                                         out_hdr, out_pitch, exposure, op, ldr, ldr_pitch);
+  if (e == cudaSuccess) {
+    auto launch = in32 ? (out32 ? launch_composite<EPBR_HDR_RGBA32F, EPBR_HDR_RGBA32F>
+                                : launch_composite<EPBR_HDR_RGBA32F, EPBR_HDR_RGBA16F>)
+                       : (out32 ? launch_composite<EPBR_HDR_RGBA16F, EPBR_HDR_RGBA32F>
+                                : launch_composite<EPBR_HDR_RGBA16F, EPBR_HDR_RGBA16F>);
+    e = launch(g, blk, s, hdr, hdr_pitch, width, height, d, params->strength, out_hdr, out_pitch, exposure, op, ldr,
+               ldr_pitch);
+  }
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return fail(EPBR_ERR_CUDA, "bloom: %s", cudaGetErrorString(e));
+  }
   if ((st = check_launch("bloom"))) return st;
   return ok();
 }
