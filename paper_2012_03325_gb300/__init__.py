@@ -33,8 +33,8 @@ def _check(st: int):
 
 
 def _stream(stream) -> int:
-    if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+    if stream is None:  # the raw handle: building a torch.cuda.Stream object takes ten times as long
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
@@ -56,16 +56,20 @@ def _flat(t: torch.Tensor, n: int, dtype, name: str) -> int:
     return t.data_ptr()
 
 
-def _image(t: torch.Tensor, H: int, W: int, channels: int | None, name: str, dtype=None) -> int:
-    """Pointer of an (H, W[, channels]) image read or written through its row pitch: at least H
-    rows of at least W texels, rows dense."""
-    _dev(t, dtype, name)
-    want = 2 if channels is None else 3
-    if t.dim() != want or t.shape[0] < H or t.shape[1] < W or (channels is not None and t.shape[2] != channels):
-        shape = (H, W) if channels is None else (H, W, channels)
-        raise ValueError(f"{name} must cover {shape}, got {tuple(t.shape)}")
-    _pitch(t, 1)
-    return t.data_ptr()
+def _plane(t: torch.Tensor, H: int, W: int, channels: int | None, name: str, dtype=None) -> tuple[int, int]:
+    """Pointer and row pitch of an (H, W[, channels]) image read or written through its pitch: at
+    least H rows of at least W texels, rows dense."""
+    ptr = _dev(t, dtype, name)
+    shape = t.shape
+    if (len(shape) != (2 if channels is None else 3) or shape[0] < H or shape[1] < W or
+            (channels is not None and shape[2] != channels)):
+        want = (H, W) if channels is None else (H, W, channels)
+        raise ValueError(f"{name} must cover {want}, got {tuple(shape)}")
+    return ptr, _pitch(t, 1)
+
+
+def _plane_or_null(t: torch.Tensor | None, H: int, W: int, channels: int | None, name: str, dtype=None):
+    return (None, 0) if t is None else _plane(t, H, W, channels, name, dtype)
 
 
 def _hdr_dtype(fmt: int):
@@ -74,12 +78,15 @@ def _hdr_dtype(fmt: int):
 
 def _pitch(t: torch.Tensor, texel_elems: int) -> int:
     """Row pitch in bytes of an (H, W[, C]) tensor whose rows are dense."""
-    if t.dim() >= 2:
-        inner = t[0].is_contiguous()
-        if not inner:
-            raise ValueError("rows of image tensors must be contiguous")
-        return t.stride(0) * t.element_size()
-    raise ValueError("image tensors need at least 2 dims")
+    stride = t.stride()
+    n = len(stride)
+    if n < 2:
+        raise ValueError("image tensors need at least 2 dims")
+    # the usual dense rows are told from their strides; t[0] would build a tensor
+    dense = stride[-1] == 1 and t.shape[0] > 0 and (n == 2 or (n == 3 and stride[1] == t.shape[2]))
+    if not dense and not t[0].is_contiguous():
+        raise ValueError("rows of image tensors must be contiguous")
+    return stride[0] * t.element_size()
 
 
 class GBuffer:
@@ -98,18 +105,18 @@ class GBuffer:
     @classmethod
     def fp32(cls, rt0: torch.Tensor, rt1: torch.Tensor, depth: torch.Tensor) -> "GBuffer":
         H, W = depth.shape
-        _image(rt0, H, W, 4, "rt0", torch.float32)
-        _image(rt1, H, W, 4, "rt1", torch.float32)
-        _image(depth, H, W, None, "depth", torch.float32)
+        _plane(rt0, H, W, 4, "rt0", torch.float32)
+        _plane(rt1, H, W, 4, "rt1", torch.float32)
+        _plane(depth, H, W, None, "depth", torch.float32)
         return cls(F.EPBR_GBUFFER_FP32, [rt0, rt1, None, depth], W, H)
 
     @classmethod
     def compact(cls, rt0: torch.Tensor, rt1: torch.Tensor, rt2: torch.Tensor, depth: torch.Tensor) -> "GBuffer":
         H, W = depth.shape
-        _image(rt0, H, W, 4, "rt0", torch.uint8)
-        _image(rt1, H, W, 2, "rt1", torch.float16)
-        _image(rt2, H, W, 2, "rt2", torch.uint8)
-        _image(depth, H, W, None, "depth", torch.float32)
+        _plane(rt0, H, W, 4, "rt0", torch.uint8)
+        _plane(rt1, H, W, 2, "rt1", torch.float16)
+        _plane(rt2, H, W, 2, "rt2", torch.uint8)
+        _plane(depth, H, W, None, "depth", torch.float32)
         return cls(F.EPBR_GBUFFER_COMPACT, [rt0, rt1, rt2, depth], W, H)
 
 
@@ -237,14 +244,14 @@ class SsaoParams:
         return ((H + s - 1) // s, (W + s - 1) // s)
 
 
-def _ao(g: GBuffer, p: SsaoParams, t: torch.Tensor, name: str) -> int:
+def _ao(g: GBuffer, p: SsaoParams, t: torch.Tensor, name: str) -> tuple[int, int]:
     Ha, Wa = p.ao_shape(g.struct.width, g.struct.height)
-    return _image(t, Ha, Wa, None, name, torch.float32)
+    return _plane(t, Ha, Wa, None, name, torch.float32)
 
 
 def epbr_ssao_raw(g: GBuffer, cam: F.epbr_camera, p: SsaoParams, ao: torch.Tensor, stream=None):
-    _check(lib().epbr_ssao_raw(C.byref(g.struct), C.byref(cam), C.byref(p.struct), _ao(g, p, ao, "ao"),
-                               _pitch(ao, 1), _stream(stream)))
+    ap, pitch = _ao(g, p, ao, "ao")
+    _check(lib().epbr_ssao_raw(C.byref(g.struct), C.byref(cam), C.byref(p.struct), ap, pitch, _stream(stream)))
 
 
 def epbr_ssao_tiled(g: GBuffer, p: SsaoParams) -> bool:
@@ -270,17 +277,20 @@ def epbr_ssao_set_tile_wait(first_wait_ns: int) -> int:
 
 
 def epbr_ssao_blur(g: GBuffer, p: SsaoParams, ao_in: torch.Tensor, ao_out: torch.Tensor, stream=None):
-    _check(lib().epbr_ssao_blur(C.byref(g.struct), C.byref(p.struct), _ao(g, p, ao_in, "ao_in"), _pitch(ao_in, 1),
-                                _ao(g, p, ao_out, "ao_out"), _pitch(ao_out, 1), _stream(stream)))
+    ip, in_pitch = _ao(g, p, ao_in, "ao_in")
+    op, out_pitch = _ao(g, p, ao_out, "ao_out")
+    _check(lib().epbr_ssao_blur(C.byref(g.struct), C.byref(p.struct), ip, in_pitch, op, out_pitch, _stream(stream)))
 
 
 def epbr_ssao(g: GBuffer, cam: F.epbr_camera, p: SsaoParams, ao: torch.Tensor, workspace=None, stream=None):
-    _ao(g, p, ao, "ao")
-    n = C.c_size_t()
-    _check(lib().epbr_ssao_workspace_size(C.byref(g.struct), C.byref(p.struct), C.byref(n)))
-    ws = workspace if workspace is not None else _workspace(n.value, ao.device)
-    _check(lib().epbr_ssao(C.byref(g.struct), C.byref(cam), C.byref(p.struct), ao.data_ptr(), _pitch(ao, 1),
-                           _aligned(ws), ws.numel() - (_aligned(ws) - ws.data_ptr()), _stream(stream)))
+    ap, pitch = _ao(g, p, ao, "ao")
+    if workspace is None:
+        n = C.c_size_t()
+        _check(lib().epbr_ssao_workspace_size(C.byref(g.struct), C.byref(p.struct), C.byref(n)))
+        workspace = _workspace(n.value, ao.device)
+    wp = _aligned(workspace)
+    _check(lib().epbr_ssao(C.byref(g.struct), C.byref(cam), C.byref(p.struct), ap, pitch, wp,
+                           workspace.numel() - (wp - workspace.data_ptr()), _stream(stream)))
 
 
 def shade_params(flags: int = EPBR_SHADE_ALL, ao: torch.Tensor | None = None, ao_scale: int = 2):
@@ -303,9 +313,9 @@ def _lights(lights: torch.Tensor | None):
 def epbr_shade(g: GBuffer, cam: F.epbr_camera, lights: torch.Tensor | None, ibl: Ibl | None,
                params: F.epbr_shade_params, hdr: torch.Tensor, hdr_format: int = EPBR_HDR_RGBA32F, stream=None):
     lp, nl = _lights(lights)
-    hp = _image(hdr, g.struct.height, g.struct.width, 4, "hdr", _hdr_dtype(hdr_format))
+    hp, hpitch = _plane(hdr, g.struct.height, g.struct.width, 4, "hdr", _hdr_dtype(hdr_format))
     _check(lib().epbr_shade(C.byref(g.struct), C.byref(cam), lp, nl, C.byref(ibl.struct) if ibl else None,
-                            C.byref(params), hp, hdr_format, _pitch(hdr, 1), _stream(stream)))
+                            C.byref(params), hp, hdr_format, hpitch, _stream(stream)))
 
 
 def epbr_shade_light_timeouts() -> int:
@@ -324,19 +334,18 @@ def epbr_shade_tonemap(g: GBuffer, cam: F.epbr_camera, lights, ibl: Ibl | None, 
                        stream=None):
     lp, nl = _lights(lights)
     H, W = g.struct.height, g.struct.width
-    dp = _image(ldr, H, W, 4, "ldr", torch.uint8)
-    hp, hpitch = (None, 0) if hdr is None else (_image(hdr, H, W, 4, "hdr", _hdr_dtype(hdr_format)), _pitch(hdr, 1))
+    dp, dpitch = _plane(ldr, H, W, 4, "ldr", torch.uint8)
+    hp, hpitch = _plane_or_null(hdr, H, W, 4, "hdr", _hdr_dtype(hdr_format))
     _check(lib().epbr_shade_tonemap(C.byref(g.struct), C.byref(cam), lp, nl, C.byref(ibl.struct) if ibl else None,
-                                    C.byref(params), hp, hdr_format, hpitch, C.byref(tp), dp,
-                                    _pitch(ldr, 1), _stream(stream)))
+                                    C.byref(params), hp, hdr_format, hpitch, C.byref(tp), dp, dpitch,
+                                    _stream(stream)))
 
 
 def epbr_tonemap(hdr: torch.Tensor, hdr_format: int, tp: F.epbr_tonemap_params, out: torch.Tensor, stream=None):
     H, W = hdr.shape[0], hdr.shape[1]
-    hp = _image(hdr, H, W, 4, "hdr", _hdr_dtype(hdr_format))
-    op = _image(out, H, W, 4, "out", torch.uint8)
-    _check(lib().epbr_tonemap(hp, hdr_format, W, H, _pitch(hdr, 1), C.byref(tp), op,
-                              _pitch(out, 1), _stream(stream)))
+    hp, hpitch = _plane(hdr, H, W, 4, "hdr", _hdr_dtype(hdr_format))
+    op, opitch = _plane(out, H, W, 4, "out", torch.uint8)
+    _check(lib().epbr_tonemap(hp, hdr_format, W, H, hpitch, C.byref(tp), op, opitch, _stream(stream)))
 
 
 # ------------------------------------------------------------------------------------------
@@ -367,10 +376,9 @@ def epbr_raster_gbuffer(mesh: Mesh, cam: F.epbr_camera, near: float, out: GBuffe
     W, H = out.struct.width, out.struct.height
     need = epbr_raster_workspace_size(mesh.struct.num_triangles, W, H)
     ws = workspace if workspace is not None else _workspace(need, mesh.tensors[0].device)
-    ip = _image(ids, H, W, None, "ids", torch.int32) if ids is not None else None
-    _check(lib().epbr_raster_gbuffer(C.byref(mesh.struct), C.byref(cam), near, C.byref(out.struct), ip,
-                                     _pitch(ids, 1) if ids is not None else 0, _aligned(ws),
-                                     ws.numel() - (_aligned(ws) - ws.data_ptr()), _stream(stream)))
+    ip, ipitch = _plane_or_null(ids, H, W, None, "ids", torch.int32)
+    _check(lib().epbr_raster_gbuffer(C.byref(mesh.struct), C.byref(cam), near, C.byref(out.struct), ip, ipitch,
+                                     _aligned(ws), ws.numel() - (_aligned(ws) - ws.data_ptr()), _stream(stream)))
 
 
 class Surfels:
@@ -395,10 +403,10 @@ def epbr_surfel_gbuffer(surfels: Surfels, cam: F.epbr_camera, near: float, toler
     W, H = out.struct.width, out.struct.height
     need = epbr_surfel_workspace_size(surfels.struct.num_surfels, W, H)
     ws = workspace if workspace is not None else _workspace(need, surfels.tensors[0].device)
-    wp = _image(weight, H, W, None, "weight", torch.float32) if weight is not None else None
+    wp, wpitch = _plane_or_null(weight, H, W, None, "weight", torch.float32)
     _check(lib().epbr_surfel_gbuffer(C.byref(surfels.struct), C.byref(cam), near, tolerance, C.byref(out.struct), wp,
-                                     _pitch(weight, 1) if weight is not None else 0, _aligned(ws),
-                                     ws.numel() - (_aligned(ws) - ws.data_ptr()), _stream(stream)))
+                                     wpitch, _aligned(ws), ws.numel() - (_aligned(ws) - ws.data_ptr()),
+                                     _stream(stream)))
 
 
 def epbr_shadow_maps_workspace_size(num_triangles: int, size: int) -> int:
@@ -433,14 +441,12 @@ def epbr_edl(g: GBuffer, params: F.epbr_edl_params, hdr: torch.Tensor | None, hd
              ao: torch.Tensor | None = None, ao_scale: int = 2, tp: F.epbr_tonemap_params | None = None,
              ldr: torch.Tensor | None = None, stream=None):
     H, W = g.struct.height, g.struct.width
-    ap = _image(ao, (H + ao_scale - 1) // ao_scale, (W + ao_scale - 1) // ao_scale, None, "ao",
-                torch.float32) if ao is not None else None
-    hp = _image(hdr, H, W, 4, "hdr", _hdr_dtype(hdr_format)) if hdr is not None else None
-    dp = _image(ldr, H, W, 4, "ldr", torch.uint8) if ldr is not None else None
-    _check(lib().epbr_edl(C.byref(g.struct), C.byref(params), ap, _pitch(ao, 1) if ao is not None else 0, ao_scale,
-                          hp, hdr_format, _pitch(hdr, 1) if hdr is not None else 0,
-                          C.byref(tp) if tp is not None else None, dp, _pitch(ldr, 1) if ldr is not None else 0,
-                          _stream(stream)))
+    ap, apitch = (None, 0) if ao is None else _plane(ao, (H + ao_scale - 1) // ao_scale, (W + ao_scale - 1) // ao_scale,
+                                                     None, "ao", torch.float32)
+    hp, hpitch = _plane_or_null(hdr, H, W, 4, "hdr", _hdr_dtype(hdr_format))
+    dp, dpitch = _plane_or_null(ldr, H, W, 4, "ldr", torch.uint8)
+    _check(lib().epbr_edl(C.byref(g.struct), C.byref(params), ap, apitch, ao_scale, hp, hdr_format, hpitch,
+                          C.byref(tp) if tp is not None else None, dp, dpitch, _stream(stream)))
 
 
 # ------------------------------------------------------------------------------------------
@@ -467,12 +473,11 @@ def epbr_shade_shadows(g: GBuffer, cam: F.epbr_camera, lights, ibl: Ibl | None, 
                        tp: F.epbr_tonemap_params | None = None, ldr: torch.Tensor | None = None, stream=None):
     lp, nl = _lights(lights)
     H, W = g.struct.height, g.struct.width
-    hp = _image(hdr, H, W, 4, "hdr", _hdr_dtype(hdr_format)) if hdr is not None else None
-    dp = _image(ldr, H, W, 4, "ldr", torch.uint8) if ldr is not None else None
+    hp, hpitch = _plane_or_null(hdr, H, W, 4, "hdr", _hdr_dtype(hdr_format))
+    dp, dpitch = _plane_or_null(ldr, H, W, 4, "ldr", torch.uint8)
     _check(lib().epbr_shade_shadows(C.byref(g.struct), C.byref(cam), lp, nl, C.byref(ibl.struct) if ibl else None,
-                                    C.byref(params), C.byref(shadows.struct), hp, hdr_format,
-                                    _pitch(hdr, 1) if hdr is not None else 0, C.byref(tp) if tp is not None else None,
-                                    dp, _pitch(ldr, 1) if ldr is not None else 0, _stream(stream)))
+                                    C.byref(params), C.byref(shadows.struct), hp, hdr_format, hpitch,
+                                    C.byref(tp) if tp is not None else None, dp, dpitch, _stream(stream)))
 
 
 # ------------------------------------------------------------------------------------------
@@ -493,15 +498,14 @@ def epbr_bloom(hdr: torch.Tensor, hdr_format: int, bp: F.epbr_bloom_params, out_
                out_format: int = EPBR_HDR_RGBA32F, tp: F.epbr_tonemap_params | None = None,
                ldr: torch.Tensor | None = None, workspace: torch.Tensor | None = None, stream=None):
     H, W = hdr.shape[0], hdr.shape[1]
-    _image(hdr, H, W, 4, "hdr", _hdr_dtype(hdr_format))
+    hp, hpitch = _plane(hdr, H, W, 4, "hdr", _hdr_dtype(hdr_format))
     need = epbr_bloom_workspace_size(W, H, bp)
     ws = workspace if workspace is not None else _workspace(need, hdr.device)
-    op = _image(out_hdr, H, W, 4, "out_hdr", _hdr_dtype(out_format)) if out_hdr is not None else None
-    lp = _image(ldr, H, W, 4, "ldr", torch.uint8) if ldr is not None else None
-    _check(lib().epbr_bloom(hdr.data_ptr(), hdr_format, _pitch(hdr, 1), W, H, C.byref(bp), _aligned(ws),
-                            ws.numel() - (_aligned(ws) - ws.data_ptr()), op, out_format,
-                            _pitch(out_hdr, 1) if out_hdr is not None else 0, C.byref(tp) if tp is not None else None,
-                            lp, _pitch(ldr, 1) if ldr is not None else 0, _stream(stream)))
+    op, opitch = _plane_or_null(out_hdr, H, W, 4, "out_hdr", _hdr_dtype(out_format))
+    lp, lpitch = _plane_or_null(ldr, H, W, 4, "ldr", torch.uint8)
+    _check(lib().epbr_bloom(hp, hdr_format, hpitch, W, H, C.byref(bp), _aligned(ws),
+                            ws.numel() - (_aligned(ws) - ws.data_ptr()), op, out_format, opitch,
+                            C.byref(tp) if tp is not None else None, lp, lpitch, _stream(stream)))
 
 
 # ------------------------------------------------------------------------------------------
@@ -513,9 +517,9 @@ def view(g: GBuffer, cam: F.epbr_camera, lights: torch.Tensor | None, ibl_index:
     v = F.epbr_view()
     v.gbuffer, v.camera, v.lights, v.num_lights, v.ibl_index = g.struct, cam, lp, nl, ibl_index
     H, W = g.struct.height, g.struct.width
-    v.ldr, v.ldr_pitch = _image(ldr, H, W, 4, "ldr", torch.uint8), _pitch(ldr, 1)
+    v.ldr, v.ldr_pitch = _plane(ldr, H, W, 4, "ldr", torch.uint8)
     if hdr is not None:
-        v.hdr, v.hdr_pitch = _image(hdr, H, W, 4, "hdr"), _pitch(hdr, 1)
+        v.hdr, v.hdr_pitch = _plane(hdr, H, W, 4, "hdr")
     return v
 
 
