@@ -145,9 +145,21 @@ __global__ void __launch_bounds__(kBloomTX* kBloomTY) k_bloom_blur(const __grid_
   b -= d.tile_start[k];
   const int by = b / tiles_x;
   const int x0 = (b - by * tiles_x) * kBlurTW, y0 = by * kBlurTH;
-  for (int ty = threadIdx.y; ty < TH; ty += kBloomTY) {
-    const float4* row = lv.pyr + (size_t)min(max(y0 - R + ty, 0), lv.H - 1) * lv.W;
-    for (int tx = threadIdx.x; tx < kBlurTW + 2 * R; tx += kBloomTX) s_in[ty][tx] = row[min(max(x0 - R + tx, 0), lv.W - 1)];
+  {
+    // all of a thread's texels are loaded before the first is stored
+    constexpr int kIn = kBlurTW + 2 * R, kTexels = TH * kIn, kThreads = kBloomTX * kBloomTY;
+    constexpr int kLoads = (kTexels + kThreads - 1) / kThreads;
+    float4 v[kLoads];
+#pragma unroll
+    for (int t = 0; t < kLoads; ++t) {
+      const int q = min(tid + t * kThreads, kTexels - 1), ty = q / kIn, tx = q - ty * kIn;
+      v[t] = lv.pyr[(size_t)min(max(y0 - R + ty, 0), lv.H - 1) * lv.W + min(max(x0 - R + tx, 0), lv.W - 1)];
+    }
+#pragma unroll
+    for (int t = 0; t < kLoads; ++t) {
+      const int q = tid + t * kThreads, ty = q / kIn, tx = q - ty * kIn;
+      if (q < kTexels) s_in[ty][tx] = v[t];
+    }
   }
   __syncthreads();
   // rows: four neighbouring outputs per thread, lanes down the rows
@@ -252,7 +264,10 @@ __device__ __forceinline__ void bloom_add_quad(const BloomDev& d, float strength
 }
 
 template <int HF, int OF, bool LDR>
-__global__ void __launch_bounds__(kBloomTX* kBloomTY)
+// Bound by latency at 4 blocks per SM (64 registers): bounds of 3, 5 and 6 blocks measured 41.0, 44.9 and
+// 46.8 us for the pass against 38.9, and the level count as a template parameter (all levels' loads
+// first, 100 registers) 44.9.
+__global__ void __launch_bounds__(kBloomTX* kBloomTY, 4)
     k_bloom_composite(const void* hdr, long long pitch, int W, int H, const __grid_constant__ BloomDev d, float strength,
                       void* out, long long out_pitch, float exposure, int op, uint8_t* ldr, long long ldr_pitch) {
   const int qi = blockIdx.x * kBloomTX + threadIdx.x, qj = blockIdx.y * kBloomTY + threadIdx.y;
