@@ -4,6 +4,7 @@
 //          their max(0, .) terms vanish), then each pixel sums its N neighbours' log-depth drops,
 //          shades its colour by exp(-A w), optionally times AO, and stores HDR and / or the
 //          tone-mapped 8-bit image.
+//   k_edl_ring  the same for the eight adjacent pixels (radius 1, 8 directions), four rows per thread
 #include <string.h>
 
 #include <cmath>
@@ -96,10 +97,100 @@ __global__ void __launch_bounds__(kEdlBX* kEdlBY)
   }
 }
 
+// The usual eight neighbours at distance 1, four vertically adjacent pixels per thread: a thread's
+// neighbourhood is 3 x 6 log depths (4.5 shared-memory reads per pixel instead of 9), the block's
+// 32 x 32 pixels with their border 1.13 logarithms per pixel instead of 1.2.  Neighbour k of the eight
+// directions lies at kRing[k], the order in which the drops are added.  Bound by DRAM latency and issue:
+// 1080p FP32 colour to RGBA32F and RGBA8 24.9 us by k_edl, 22.1 us here with the depths staged first and
+// the colours read after them, 18.9 us (4.4 TB/s) with a thread's depths and colours requested together.
+constexpr int kRingTileH = 32;
+__device__ constexpr int kRingX[8] = {1, 1, 0, -1, -1, -1, 0, 1}, kRingY[8] = {0, 1, 1, 1, 0, -1, -1, -1};
+
+template <int FMT, int HDR, bool LDR>
+__global__ void __launch_bounds__(kEdlBX* kEdlBY)
+    k_edl_ring(GbufDev g, const __grid_constant__ EdlDev p, void* hdr, long long hdr_pitch, float exposure, int op,
+               uint8_t* ldr, long long ldr_pitch) {
+  constexpr int TW = kEdlBX + 2, TH = kRingTileH + 2;
+  __shared__ float s_l[TH * TW];
+  const int tid = threadIdx.y * kEdlBX + threadIdx.x;
+  const int x0 = blockIdx.x * kEdlBX, y0 = blockIdx.y * kRingTileH;
+  const int x = x0 + threadIdx.x, ya = y0 + 4 * threadIdx.y;
+  const float inf = __int_as_float(0x7f800000);
+  auto depth_at = [&](int xx, int yy) {  // off the image: no surface
+    return (unsigned)xx < (unsigned)g.W && (unsigned)yy < (unsigned)g.H
+               ? __ldg((const float*)(g.rt[3] + (long long)yy * g.pitch[3]) + xx)
+               : inf;
+  };
+  // the border: rows -1 and 32, then columns -1 and 32, a texel for each of the first 132 threads
+  int bx = 0, by = 0;
+  if (tid < 2 * TW) {
+    by = tid < TW ? 0 : TH - 1;
+    bx = tid < TW ? tid : tid - TW;
+  } else {
+    by = 1 + ((tid - 2 * TW) >> 1);
+    bx = (tid & 1) ? TW - 1 : 0;  // 2 TW is even
+  }
+  const bool border = tid < 2 * TW + 2 * kRingTileH;
+  // everything a thread reads is requested at once: its pixels' depths and colours (also of
+  // background pixels, which the shading below ignores) and its border texel
+  float e[4], eb = inf;
+  float3 col[4];
+#pragma unroll
+  for (int h = 0; h < 4; ++h) {
+    e[h] = depth_at(x, ya + h);
+    col[h] = f3(0, 0, 0);
+    if (x < g.W && ya + h < g.H) col[h] = edl_colour<FMT>(g, x, ya + h);
+  }
+  if (border) eb = depth_at(x0 - 1 + bx, y0 - 1 + by);
+  auto log_of = [&](float d) { return is_surface(d) ? lg2_ftz(d) : inf; };
+  float* mine = s_l + (4 * threadIdx.y + 1) * TW + threadIdx.x + 1;
+#pragma unroll
+  for (int h = 0; h < 4; ++h) mine[h * TW] = log_of(e[h]);
+  if (border) s_l[by * TW + bx] = log_of(eb);
+  __syncthreads();
+  if (x >= g.W) return;
+  float v[6][3];
+  const float* at = s_l + 4 * threadIdx.y * TW + threadIdx.x;
+#pragma unroll
+  for (int r = 0; r < 6; ++r)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) v[r][c] = at[r * TW + c];
+#pragma unroll
+  for (int h = 0; h < 4; ++h) {
+    const int y = ya + h;
+    if (y >= g.H) continue;
+    const float lp = v[h + 1][1];
+    float3 c = f3(0, 0, 0);
+    if (lp != inf) {
+      float w = 0.0f;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) w += fmaxf(lp - v[h + 1 + kRingY[k]][1 + kRingX[k]], 0.0f);
+      float shade = ex2_ftz(p.minus_a_log2e * (w * p.inv_n));
+      if (p.ao)
+        shade *= __ldg((const float*)((const char*)p.ao + (size_t)__float2int_rd(((float)y + 0.5f) * p.ao_inv) *
+                                                              p.ao_pitch) +
+                       __float2int_rd(((float)x + 0.5f) * p.ao_inv));
+      c = col[h] * shade;
+    }
+    if (hdr) store_hdr<HDR>(hdr, hdr_pitch, x, y, c);
+    if (LDR) ((unsigned*)(ldr + (size_t)y * ldr_pitch))[x] = pack_rgba8(c, exposure, op);
+  }
+}
+
+static const int kRingHost[8][2] = {{1, 0}, {1, 1}, {0, 1}, {-1, 1}, {-1, 0}, {-1, -1}, {0, -1}, {1, -1}};
+
 template <int FMT, int HDR>
 static void launch_edl(dim3 grd, dim3 blk, cudaStream_t s, const GbufDev& g, const EdlDev& p, void* hdr,
                        long long hp, float exposure, int op, uint8_t* ldr, long long lp) {
-  if (p.N == 8) {  // the usual eight directions: neighbour loop unrolled
+  bool ring = p.N == 8;
+  for (int k = 0; k < 8; ++k) ring = ring && p.dx[k] == kRingHost[k][0] && p.dy[k] == kRingHost[k][1];
+  if (ring) {
+    grd.y = (g.H + kRingTileH - 1) / kRingTileH;
+    if (ldr)
+      k_edl_ring<FMT, HDR, true><<<grd, blk, 0, s>>>(g, p, hdr, hp, exposure, op, ldr, lp);
+    else
+      k_edl_ring<FMT, HDR, false><<<grd, blk, 0, s>>>(g, p, hdr, hp, exposure, op, ldr, lp);
+  } else if (p.N == 8) {  // eight directions: neighbour loop unrolled
     if (ldr)
       k_edl<FMT, HDR, true, 8><<<grd, blk, 0, s>>>(g, p, hdr, hp, exposure, op, ldr, lp);
     else
