@@ -1,7 +1,7 @@
 // Per-pixel compose as device functions, shared by the per-view kernel (shade.cu) and the fused
 // multi-view kernel (batch.cu):
 //   px_setup     G-buffer decode (Table 1 layouts), position from depth (Sec. 4), material terms
-//   px_direct    Cook-Torrance over a chunk of point lights staged in shared memory (Sec. 3,
+//   px_direct*   Cook-Torrance over a chunk of point lights staged in shared memory (Sec. 3,
 //                Eq. 1 with the UE4 model)
 //   px_ambient   split-sum IBL with multiple-scattering compensation, times AO (Sec. 3.1)
 //   tonemap      ACES / Reinhard + sRGB transfer (Sec. 5.4)
@@ -268,45 +268,6 @@ __device__ __forceinline__ LightTerms light_terms(const Px& s, const Direct& d, 
   return t;
 }
 
-// Adds `cnt` staged lights with arbitrary colours.
-__device__ __forceinline__ void px_direct(const Px& s, Direct& d, const float4* s_lights, int cnt) {
-  float3 sa = d.sa, sb = d.sb, sbf = d.sbf;
-#pragma unroll 4
-  for (int i = 0; i < cnt; ++i) {
-    float4 lc = s_lights[2 * i + 1];
-    LightTerms t = light_terms(s, d, s_lights[2 * i]);
-    sa.x = fmaf(lc.x, t.a, sa.x);
-    sa.y = fmaf(lc.y, t.a, sa.y);
-    sa.z = fmaf(lc.z, t.a, sa.z);
-    sb.x = fmaf(lc.x, t.b, sb.x);
-    sb.y = fmaf(lc.y, t.b, sb.y);
-    sb.z = fmaf(lc.z, t.b, sb.z);
-    sbf.x = fmaf(lc.x, t.bf, sbf.x);
-    sbf.y = fmaf(lc.y, t.bf, sbf.y);
-    sbf.z = fmaf(lc.z, t.bf, sbf.z);
-  }
-  d.sa = sa;
-  d.sb = sb;
-  d.sbf = sbf;
-}
-
-// Adds `cnt` staged monochrome lights (Ic_r = Ic_g = Ic_b).
-__device__ __forceinline__ void px_direct_mono(const Px& s, Direct& d, const float4* s_lights, int cnt) {
-  float sa = 0.0f, sb = 0.0f, sbf = 0.0f;
-#pragma unroll(kLightUnroll)
-  for (int i = 0; i < cnt; ++i) {
-    float4 lp = s_lights[2 * i];
-    float ic = lp.w;
-    LightTerms t = light_terms(s, d, lp);
-    sa = fmaf(ic, t.a, sa);
-    sb = fmaf(ic, t.b, sb);
-    sbf = fmaf(ic, t.bf, sbf);
-  }
-  d.sa = d.sa + f3(sa, sa, sa);
-  d.sb = d.sb + f3(sb, sb, sb);
-  d.sbf = d.sbf + f3(sbf, sbf, sbf);
-}
-
 // alpha^2 G1(v) / (4 pi n.v): the per-pixel factor of the specular sums.
 __device__ __forceinline__ float spec_factor(const Px& s) {
   float alpha = s.rough * s.rough, k = (s.rough + 1.0f) * (s.rough + 1.0f) * 0.125f;
@@ -449,6 +410,86 @@ __device__ __forceinline__ void px_direct_mono2(const Frame2& f, Sums2& S, const
   S.w = sw, S.wf = swf, S.b = sb, S.bf = sbf;
 }
 
+// light_terms for two (pixel, light) pairs at once, step by step the same arithmetic with each step
+// one packed FP32x2 instruction, so each half is light_terms' result bit for bit.
+struct Geo2 {  // per pair: unit normal, its negative, unit view vector, alpha n.v, alpha, k, 1 - k
+  float2 nx, ny, nz, mnx, mny, mnz, vx, vy, vz, nva, alpha, k, omk;
+};
+struct Terms2 {
+  float2 a, b, bf;
+};
+
+__device__ __forceinline__ Terms2 light_terms2(const Geo2& g, float2 Lx, float2 Ly, float2 Lz) {
+  const float2 e30 = dup2(1e-30f), e18 = dup2(1e-18f), mhalf = dup2(-0.5f), one = dup2(1.0f), minus = dup2(-1.0f);
+  const float2 d2 = pfma(Lx, Lx, pfma(Ly, Ly, pfma(Lz, Lz, e30)));
+  const float2 rs = make_float2(rsqrt_ftz(d2.x), rsqrt_ftz(d2.y));
+  const float2 lx = pmul(Lx, rs), ly = pmul(Ly, rs), lz = pmul(Lz, rs);
+  const float2 nl = pfma(g.nx, lx, pfma(g.ny, ly, pmul(g.nz, lz)));
+  const float2 nlc = make_float2(fmaxf(nl.x, 0.0f), fmaxf(nl.y, 0.0f));
+  const float2 hx = pfma(Lx, rs, g.vx), hy = pfma(Ly, rs, g.vy), hz = pfma(Lz, rs, g.vz);  // s = l + v
+  const float2 cx = pfma(g.ny, hz, pmul(g.mnz, hy)), cy = pfma(g.nz, hx, pmul(g.mnx, hz)),
+               cz = pfma(g.nx, hy, pmul(g.mny, hx));
+  const float2 c2 = pfma(cx, cx, pfma(cy, cy, pfma(cz, cz, e18)));
+  const float2 nsa = pfma(nl, g.alpha, g.nva);
+  const float2 hh = pfma(hx, hx, pfma(hy, hy, pmul(hz, hz)));
+  const float2 den = pfma(nsa, nsa, c2);
+  const float2 xx = pfma(mhalf, make_float2(sqrt_ftz(hh.x), sqrt_ftz(hh.y)), one);
+  const float2 fc = make_float2(ex2_ftz(5.0f * lg2_ftz(fabsf(xx.x))), ex2_ftz(5.0f * lg2_ftz(fabsf(xx.y))));
+  const float2 w = pmul(pmul(rs, rs), nlc);
+  const float2 q = pmul(pmul(den, den), pfma(nlc, g.omk, g.k));
+  const float2 spec = pmul(pmul(hh, hh), make_float2(rcp_ftz(q.x), rcp_ftz(q.y)));
+  const float2 b = pmul(w, spec);
+  return Terms2{pfma(pmul(w, minus), fc, w), b, pmul(b, fc)};
+}
+
+// Adds `cnt` lights of arbitrary colours (staged as for px_direct_mono2, colours in s_lights) to both
+// pixels' sums, bit for bit those of a loop over one pixel's light_terms (three FMAs per sum and
+// light).  An inactive half computes finite values that are never used.  Half the issue slots of that
+// loop: a 1283 x 721 frame with 12 coloured lights 67.4 -> 65.5 us.
+struct Direct2 {
+  float2 sa[3], sb[3], sbf[3];
+};
+
+__device__ __forceinline__ Direct2 px_direct2(const Px (&s)[2], const bool (&act)[2], const float4* s_lights,
+                                              const float4* s_dup, int cnt) {
+  float c[2][15];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+#pragma unroll
+    for (int q = 0; q < 15; ++q) c[h][q] = q >= 11 ? 1.0f : 0.0f;
+    if (!act[h]) continue;
+    const Direct d = px_direct_begin(s[h]);
+    const float v[15] = {-s[h].P.x, -s[h].P.y, -s[h].P.z, s[h].n.x, s[h].n.y, s[h].n.z, s[h].v.x, s[h].v.y,
+                         s[h].v.z, d.nva, 0.0f, d.alpha, d.k, d.omk, 0.0f};
+#pragma unroll
+    for (int q = 0; q < 15; ++q) c[h][q] = v[q];
+  }
+  auto two = [&](int q) { return make_float2(c[0][q], c[1][q]); };
+  const float2 mPx = two(0), mPy = two(1), mPz = two(2);
+  Geo2 g;
+  g.nx = two(3), g.ny = two(4), g.nz = two(5), g.vx = two(6), g.vy = two(7), g.vz = two(8);
+  g.nva = two(9), g.alpha = two(11), g.k = two(12), g.omk = two(13);
+  g.mnx = make_float2(-g.nx.x, -g.nx.y), g.mny = make_float2(-g.ny.x, -g.ny.y), g.mnz = make_float2(-g.nz.x, -g.nz.y);
+  Direct2 D;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) D.sa[q] = D.sb[q] = D.sbf[q] = make_float2(0.0f, 0.0f);
+#pragma unroll 1  // more lights at a time spill in the multi-view kernel and are no faster
+  for (int i = 0; i < cnt; ++i) {
+    const float4 u = s_dup[2 * i], z = s_dup[2 * i + 1], lc = s_lights[2 * i + 1];
+    const Terms2 t = light_terms2(g, padd(make_float2(u.x, u.y), mPx), padd(make_float2(u.z, u.w), mPy),
+                                  padd(make_float2(z.x, z.y), mPz));
+    const float ic[3] = {lc.x, lc.y, lc.z};
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      const float2 I = dup2(ic[r]);
+      D.sa[r] = pfma(I, t.a, D.sa[r]);
+      D.sb[r] = pfma(I, t.b, D.sb[r]);
+      D.sbf[r] = pfma(I, t.bf, D.sbf[r]);
+    }
+  }
+  return D;
+}
+
 // Folds half `h` (0 or 1) of the packed sums into pixel s.
 __device__ __forceinline__ void px_direct_fold2(Px& s, const Sums2& S, int h) {
   float w = h ? S.w.y : S.w.x, wf = h ? S.wf.y : S.wf.x, b = h ? S.b.y : S.b.x, bf = h ? S.bf.y : S.bf.x;
@@ -466,10 +507,17 @@ __device__ __forceinline__ void shade_lights(Px (&s)[2], const bool (&act)[2], i
                                              const float4* __restrict__ lights, float4* s_lights, float4* s_dup,
                                              int chunk, bool prestaged, bool mono, int tid, int nthreads) {
   const bool diffuse_only = (flags & EPBR_SHADE_DIFFUSE_ONLY) != 0;
-  Frame2 fr;
   Sums2 sums;
   sums.w = sums.wf = sums.b = sums.bf = make_float2(0.0f, 0.0f);
-  if (NL > 0 && !diffuse_only && (act[0] || act[1])) fr = make_frame2(s[0], act[0], s[1], act[1]);
+  if (prestaged && mono && !diffuse_only) {  // the usual case by itself, so that no other loop's registers weigh on it
+    if (NL == 0 || !(act[0] || act[1])) return;
+    const Frame2 fr = make_frame2(s[0], act[0], s[1], act[1]);
+    px_direct_mono2(fr, sums, s_dup, NL);
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (act[h]) px_direct_fold2(s[h], sums, h);
+    return;
+  }
   for (int base = 0; base < NL; base += chunk) {
     int cnt = prestaged ? NL : min(chunk, NL - base);
     bool m = mono;
@@ -478,21 +526,25 @@ __device__ __forceinline__ void shade_lights(Px (&s)[2], const bool (&act)[2], i
       m = __syncthreads_and(stage_lights(s_lights, lights, base, cnt, tid, nthreads, s_dup));
     }
     if (!(act[0] || act[1])) continue;
-    if (!diffuse_only && m) {
-      px_direct_mono2(fr, sums, s_dup, cnt);
+    if (!diffuse_only && m) {  // the frames per chunk: not held in registers over the other loops
+      px_direct_mono2(make_frame2(s[0], act[0], s[1], act[1]), sums, s_dup, cnt);
+      continue;
+    }
+    if (!diffuse_only) {
+      const Direct2 D = px_direct2(s, act, s_lights, s_dup, cnt);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        auto half = [h](const float2 (&v)[3]) { return h ? f3(v[0].y, v[1].y, v[2].y) : f3(v[0].x, v[1].x, v[2].x); };
+        if (act[h]) px_direct_fold(s[h], half(D.sa), half(D.sb), half(D.sbf), px_direct_begin(s[h]).a2vv);
+      }
       continue;
     }
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       if (!act[h]) continue;
       Direct d = px_direct_begin(s[h]);
-      if (diffuse_only) {
-        px_direct_diffuse(s[h], d, s_lights, cnt);
-        px_direct_diffuse_end(s[h], d);
-      } else {
-        px_direct(s[h], d, s_lights, cnt);
-        px_direct_end(s[h], d);
-      }
+      px_direct_diffuse(s[h], d, s_lights, cnt);
+      px_direct_diffuse_end(s[h], d);
     }
   }
   if (NL > 0 && !diffuse_only) {
