@@ -1,7 +1,8 @@
 // Shadow maps with 3x3 percentage-closer filtering for the point lights (Sec. 5.1; Williams
 // 1978, Reeves et al. 1987), evaluated inside the compose's light loop.
-//   k_shade_shadow  one pixel per thread in 32x8 blocks, lights and their shadow cameras staged
-//                   in shared memory in chunks of 128; per light the direct terms of Eq. 1 and,
+//   k_shade_shadow  one pixel per thread in 32x4 blocks, lights and their shadow cameras staged
+//                   in shared memory in chunks of 128; per light (monochrome lights two at a time in
+//                   packed FP32x2 arithmetic, the same bits) the direct terms of Eq. 1 and,
 //                   when the light reaches the pixel (n.l > 0), its PCF visibility: the fragment
 //                   projected into the light's map and the 3x3 block of depths around its texel
 //                   compared with z - b0 - b1 z.  Ambient, background and tone map as k_shade.
@@ -67,15 +68,65 @@ __device__ __forceinline__ float shadow_visibility(const float4* cam, float3 P, 
   return (float)lit * (1.0f / 9.0f);
 }
 
+// Two lights' shadow cameras, value by value next to each other for packed arithmetic on -P: rows 0
+// (negated rotation), 1 and 2 (negated offset) of world -> light view, so that -P gives q.x, -q.y and
+// z = -q.z with the products and sums of shadow_visibility, then f.
+struct CamPair {
+  float2 r[3][4];
+  float2 f, pad;
+};
+
+// shadow_visibility of P for two lights; the taps of both are under way together where both blocks
+// lie inside their maps.
+__device__ __forceinline__ float2 shadow_visibility2(const CamPair& c, const float4* cams, const float3& P, float2 mPx,
+                                                     float2 mPy, float2 mPz, const float* __restrict__ map0,
+                                                     const float* __restrict__ map1, int S, float b0, float b1) {
+  const float2 qx = pfma(c.r[0][0], mPx, pfma(c.r[0][1], mPy, pfma(c.r[0][2], mPz, c.r[0][3])));
+  const float2 mqy = pfma(c.r[1][0], mPx, pfma(c.r[1][1], mPy, pfma(c.r[1][2], mPz, c.r[1][3])));
+  const float2 z = pfma(c.r[2][0], mPx, pfma(c.r[2][1], mPy, pfma(c.r[2][2], mPz, c.r[2][3])));
+  const float2 half = dup2(0.5f * (float)S), k = pmul(c.f, make_float2(rcp_ftz(z.x), rcp_ftz(z.y)));
+  const float2 s = pfma(pmul(qx, k), half, half), t = pfma(pmul(mqy, k), half, half);
+  const float2 thr = padd(pfma(dup2(-b1), z, z), dup2(-b0));
+  // a coordinate beyond +-1e9 converts to a texel outside the map as well
+  const int i0 = __float2int_rd(s.x), j0 = __float2int_rd(t.x), i1 = __float2int_rd(s.y), j1 = __float2int_rd(t.y);
+  const unsigned inner = (unsigned)max(S - 2, 0);
+  const bool in0 = z.x > 0.0f && (unsigned)i0 - 1u < inner && (unsigned)j0 - 1u < inner;
+  const bool in1 = z.y > 0.0f && (unsigned)i1 - 1u < inner && (unsigned)j1 - 1u < inner;
+  if (in0 && in1) {
+    const float* p = map0 + ((j0 - 1) * S + (i0 - 1));
+    const float* q = map1 + ((j1 - 1) * S + (i1 - 1));
+    float d[2][9];
+#pragma unroll
+    for (int r = 0; r < 3; ++r, p += S, q += S)
+#pragma unroll
+      for (int x = 0; x < 3; ++x) d[0][3 * r + x] = __ldg(p + x), d[1][3 * r + x] = __ldg(q + x);
+    float l0 = 0.0f, l1 = 0.0f;
+#pragma unroll
+    for (int x = 0; x < 9; ++x) {
+      l0 += d[0][x] >= thr.x ? 1.0f : 0.0f;
+      l1 += d[1][x] >= thr.y ? 1.0f : 0.0f;
+    }
+    return make_float2(l0 * (1.0f / 9.0f), l1 * (1.0f / 9.0f));
+  }
+  return make_float2(shadow_visibility(cams, P, map0, S, b0, b1), shadow_visibility(cams + 4, P, map1, S, b0, b1));
+}
+
+// 128 threads, six blocks per SM (80 registers, no spill).  Bound by issue and the LSU data pipe (ncu: 68%
+// and 59%; 459 M warp instructions, 565 M with one light at a time): 1080p with 64 lights and 512^2 maps
+// 577 us one light at a time, 547 us two at a time; 256 threads at 64 (spills), 80 and 96 registers
+// 552, 561 and 680 us, and the taps requested before the light terms 589 us at best.
+constexpr int kShadowBY = 4, kShadowThreads = 32 * kShadowBY;
 template <int FMT, int HDR, bool LDR>
-__global__ void __launch_bounds__(256, 4)
+__global__ void __launch_bounds__(kShadowThreads, 6)
     k_shade_shadow(GbufDev g, CamDev cam, const float4* __restrict__ lights, int NL, IblDev ibl, ShadeDev p,
                    ShadowDev sh, void* hdr, long long hdr_pitch, uint8_t* ldr, long long ldr_pitch) {
   __shared__ float4 s_lights[2 * kShadowChunk];
   __shared__ float4 s_cams[4 * kShadowChunk];
+  __shared__ float4 s_pos[kShadowChunk];  // per light pair (x, x, y, y), (z, z, Ic, Ic)
+  __shared__ __align__(16) CamPair s_pair[kShadowChunk / 2];
   const int tid = threadIdx.y * 32 + threadIdx.x;
   const int by = gridDim.y - 1 - blockIdx.y;  // costliest rows first, as k_shade
-  const int x = blockIdx.x * 32 + threadIdx.x, y = by * 8 + threadIdx.y;
+  const int x = blockIdx.x * 32 + threadIdx.x, y = by * kShadowBY + threadIdx.y;
   const bool inside = x < g.W && y < g.H;
   Px s;
   if (inside) s = px_setup<FMT>(g, cam, x, y);
@@ -86,14 +137,59 @@ __global__ void __launch_bounds__(256, 4)
   for (int base = 0; base < NL; base += kShadowChunk) {
     const int cnt = min(kShadowChunk, NL - base);
     __syncthreads();  // the previous chunk has been read
-    for (int q = tid; q < 4 * cnt; q += 256) s_cams[q] = __ldg(sh.cams + 4 * (size_t)base + q);
+    for (int q = tid; q < 4 * cnt; q += kShadowThreads) s_cams[q] = __ldg(sh.cams + 4 * (size_t)base + q);
     // a chunk of monochrome lights keeps one sum per kind (each channel's sum would be the same)
-    const bool mono = __syncthreads_and(stage_lights(s_lights, lights, base, cnt, tid, 256));
+    const bool mono = __syncthreads_and(stage_lights(s_lights, lights, base, cnt, tid, kShadowThreads));
+    if (mono && !diffuse_only) {  // block-uniform
+      for (int q = tid; q < cnt / 2; q += kShadowThreads) {
+        const float4 a = s_lights[4 * q], b = s_lights[4 * q + 2];
+        s_pos[2 * q] = make_float4(a.x, b.x, a.y, b.y);
+        s_pos[2 * q + 1] = make_float4(a.z, b.z, a.w, b.w);
+      }
+      for (int q = tid; q < cnt / 2 * 4; q += kShadowThreads) {
+        const int r = q & 3;
+        const float4 a = s_cams[8 * (q >> 2) + r], b = s_cams[8 * (q >> 2) + 4 + r];
+        CamPair& c = s_pair[q >> 2];
+        if (r == 3) {
+          c.f = make_float2(a.x, b.x);
+        } else {
+          const float rot = r == 0 ? -1.0f : 1.0f;  // sign changes only: exact
+          c.r[r][0] = make_float2(rot * a.x, rot * b.x);
+          c.r[r][1] = make_float2(rot * a.y, rot * b.y);
+          c.r[r][2] = make_float2(rot * a.z, rot * b.z);
+          c.r[r][3] = make_float2(-rot * a.w, -rot * b.w);
+        }
+      }
+      __syncthreads();
+    }
     if (!active) continue;
     if (mono && !diffuse_only) {
       float sa = 0.0f, sb = 0.0f, sbf = 0.0f;
       const float* map = sh.maps + (size_t)base * sh.map_texels;
-      for (int i = 0; i < cnt; ++i, map += sh.map_texels) {
+      Geo2 g;
+      g.nx = dup2(s.n.x), g.ny = dup2(s.n.y), g.nz = dup2(s.n.z);
+      g.mnx = dup2(-s.n.x), g.mny = dup2(-s.n.y), g.mnz = dup2(-s.n.z);
+      g.vx = dup2(s.v.x), g.vy = dup2(s.v.y), g.vz = dup2(s.v.z);
+      g.nva = dup2(d.nva), g.alpha = dup2(d.alpha), g.k = dup2(d.k), g.omk = dup2(d.omk);
+      const float2 mPx = dup2(-s.P.x), mPy = dup2(-s.P.y), mPz = dup2(-s.P.z);
+      int i = 0;
+      for (; i + 1 < cnt; i += 2, map += 2 * sh.map_texels) {  // two lights at a time
+        const float4 u = s_pos[i], z = s_pos[i + 1];
+        Terms2 t = light_terms2(g, padd(make_float2(u.x, u.y), mPx), padd(make_float2(u.z, u.w), mPy),
+                                padd(make_float2(z.x, z.y), mPz));
+        // the visibility (1 or less, finite) leaves the zero terms of an unlit light as they are
+        if (t.a.x > 0.0f || t.b.x > 0.0f || t.a.y > 0.0f || t.b.y > 0.0f) {
+          const float2 v = shadow_visibility2(s_pair[i >> 1], s_cams + 4 * i, s.P, mPx, mPy, mPz, map,
+                                              map + sh.map_texels, sh.S, sh.b0, sh.b1);
+          t.a = pmul(t.a, v);
+          t.b = pmul(t.b, v);
+          t.bf = pmul(t.bf, v);
+        }
+        sa = fmaf(z.w, t.a.y, fmaf(z.z, t.a.x, sa));
+        sb = fmaf(z.w, t.b.y, fmaf(z.z, t.b.x, sb));
+        sbf = fmaf(z.w, t.bf.y, fmaf(z.z, t.bf.x, sbf));
+      }
+      for (; i < cnt; ++i, map += sh.map_texels) {
         const float4 lp = s_lights[2 * i];
         LightTerms t = light_terms(s, d, lp);
         if (t.a > 0.0f || t.b > 0.0f) {
@@ -176,7 +272,7 @@ epbr_status launch_shade_shadows(const GbufDev& g, const CamDev& c, int fmt, con
                 "negative / non-finite bias");
   ShadowDev sh{s->maps, (const float4*)s->cameras, (long long)s->size * s->size, s->size, s->bias_const,
                s->bias_slope};
-  dim3 blk(32, 8), grd((g.W + 31) / 32, (g.H + 7) / 8);
+  dim3 blk(32, kShadowBY), grd((g.W + 31) / 32, (g.H + kShadowBY - 1) / kShadowBY);
   cudaError_t e;
   if (fmt == EPBR_GBUFFER_FP32) {
     if (hdr_format == EPBR_HDR_RGBA32F)
