@@ -268,18 +268,21 @@ constexpr int kSurfelTileWarps = 4;  // a block covers 4 x 1 tiles: 32 x 4 pixel
 // A warp's shared memory: up to 32 surfels of its tile.  Row strides of 80 and 48 bytes keep the
 // 16-byte reads of eight different rows free of bank conflicts, 33 words the per-pixel depths.
 struct SurfelWarp {
-  float frame[32][20];  // SurfelFrame: n, t, b, (cb, nc)
+  float frame[32][20];  // SurfelFrame: n, t, b, (cb, nc), then the packed items, a row per surfel with any
   float mat[32][12];    // world normal and metal, albedo and rough
   float depth[32][33];  // [pixel][surfel]: depth of the hits
   unsigned hits[32];    // per pixel: the surfels that cover it
   unsigned nearest[32];  // per pixel: bits of the smallest depth so far
+  float2 ray[32];        // per pixel: (ux, uy)
 };
 
 // Replaces two coverage passes of global atomics (an atomicMin, then two float4 and one float atomic
 // add per covered pixel, 13.5 M of them in the 1.2 M-surfel 1080p scene), their set-up store, resets
-// and resolve: 630 -> 265 us for the whole pass.  Bound by issue and latency at 6 blocks per SM (34 KB of
-// shared memory, 74 registers; ncu: 116 M warp instructions, 0.52 per scheduler and cycle; long
-// scoreboard 2.4, fixed latency 2.1, short scoreboard 1.9 per issue).  Blocks of 1, 2, 4, 5 warps
+// and resolve: 627 -> 256 us for the whole pass.  Bound by issue and latency at 6 blocks per SM (35 KB of
+// shared memory, 79 registers; ncu before the surfels with items took consecutive rows, an item's
+// surfel and ray then coming from nine shuffles, 269 us: 124 M warp instructions, 0.54 per scheduler
+// and cycle; long scoreboard 2.4, fixed latency 2.1, short scoreboard 1.9 per issue).  Blocks of 1, 2, 4, 5
+// warps then
 // measured 307, 294, 279, 300 us, and a lane per pixel testing every listed surfel 563 us (tiles with
 // 2000 small surfels then take the launch's tail).
 __global__ void __launch_bounds__(32 * kSurfelTileWarps)
@@ -304,6 +307,7 @@ __global__ void __launch_bounds__(32 * kSurfelTileWarps)
   }
   const float inf = __int_as_float(0x7f800000);
   st.nearest[lane] = 0xffffffffu;
+  st.ray[lane] = make_float2(ux, uy);
   // nearest depth so far and the window's end below it, the farthest blended depth, the sums
   float dmin = inf, lim = inf, far = 0.0f, w = 0.0f;
   float a0 = 0, a1 = 0, a2 = 0, a3 = 0, n0 = 0, n1 = 0, n2 = 0, n3 = 0;
@@ -334,49 +338,49 @@ __global__ void __launch_bounds__(32 * kSurfelTileWarps)
           const int v = __shfl_up_sync(0xffffffffu, incl, o);
           if (lane >= o) incl += v;
         }
-        const int total = __shfl_sync(0xffffffffu, incl, 31);
-        if (total == 0) continue;
+        const unsigned live = __ballot_sync(0xffffffffu, mine > 0);
+        if (live == 0u) continue;
+        const int total = __shfl_sync(0xffffffffu, incl, 31), excl = incl - mine;
         if (mine > 0) {
           const float4 r0 = __ldg(rec + 4 * (size_t)idx), r1 = __ldg(rec + 4 * (size_t)idx + 1);
           const float4 r2 = __ldg(rec + 4 * (size_t)idx + 2), r3 = __ldg(rec + 4 * (size_t)idx + 3);
           SurfelFrame s;
           float c[3];
           surfel_frame(r0, r1, r2, cam, s, c);
-          float4* f = (float4*)st.frame[lane];
-          f[0] = s.n, f[1] = s.t, f[2] = s.b;
-          *(float2*)(f + 3) = make_float2(s.cb, s.nc);
+          // the surfels with items, in consecutive rows; packed: clipped origin, width, its reciprocal
+          // (exact quotients of items below 32 by widths up to 8) and the first item (below 1024)
+          const int row = __popc(live & ((1u << lane) - 1u));
+          const unsigned items = (unsigned)cx | ((unsigned)cy << 3) | ((unsigned)cw << 5) |
+                                 (((255u + cw) / (unsigned)cw) << 9) | ((unsigned)excl << 18);
+          float4* f = (float4*)st.frame[row];
+          f[0] = s.n, f[1] = s.t, f[2] = s.b, f[3] = make_float4(s.cb, s.nc, __uint_as_float(items), 0.0f);
           const float rw = rsqrtf(fmaf(r1.x, r1.x, fmaf(r1.y, r1.y, r1.z * r1.z)));
-          float4* m = (float4*)st.mat[lane];
+          float4* m = (float4*)st.mat[row];
           m[0] = make_float4(r1.x * rw, r1.y * rw, r1.z * rw, r2.w);
           m[1] = r3;
         }
         st.hits[lane] = 0u;
-        // packed for the item lanes: first item, clipped origin, width and its reciprocal (exact
-        // quotients of items below 32 by widths up to 8)
-        const unsigned meta = (unsigned)cx | ((unsigned)cy << 3) | ((unsigned)cw << 5) |
-                              ((cw > 0 ? (255u + cw) / (unsigned)cw : 0u) << 9);
-        const int excl = incl - mine;
         __syncwarp();
         // a lane per (surfel, box pixel)
+        int begun = -1;  // rows whose items begin before j0, less one
         for (int j0 = 0; j0 < total; j0 += 32) {
           const int j = j0 + lane;
-          int k = 0;  // the surfels whose items end at or before j
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1)
-            if (__shfl_sync(0xffffffffu, incl, k + o - 1) <= j) k += o;
-          k = min(k, 31);
-          const unsigned m = __shfl_sync(0xffffffffu, meta, k);
-          const int local = j - __shfl_sync(0xffffffffu, excl, k);
-          const int ly = (local * (int)(m >> 9)) >> 8, lx = local - ly * (int)((m >> 5) & 15u);
-          const int px = ((int)((m >> 3) & 3u) + ly) * kTileW + (int)(m & 7u) + lx;
-          const float pux = __shfl_sync(0xffffffffu, ux, px & 31), puy = __shfl_sync(0xffffffffu, uy, px & 31);
+          const unsigned at = (unsigned)(excl - j0);
+          const unsigned begins = __reduce_or_sync(0xffffffffu, mine > 0 && at < 32u ? 1u << at : 0u);
+          const int k = begun + __popc(begins & ((2u << lane) - 1u));  // the row whose items hold j
+          begun += __popc(begins);
           if (j < total) {
             const float4* f = (const float4*)st.frame[k];
+            const float4 q = f[3];
+            const unsigned m = __float_as_uint(q.z);
+            const int local = j - (int)(m >> 18);
+            const int ly = (local * (int)((m >> 9) & 511u)) >> 8, lx = local - ly * (int)((m >> 5) & 15u);
+            const int px = ((int)((m >> 3) & 3u) + ly) * kTileW + (int)(m & 7u) + lx;
+            const float2 ray = st.ray[px];
             SurfelFrame s;
             s.n = f[0], s.t = f[1], s.b = f[2];
-            const float2 cn = *(const float2*)(f + 3);
-            s.cb = cn.x, s.nc = cn.y;
-            const float sd = surfel_hit(s, pux, puy);
+            s.cb = q.x, s.nc = q.y;
+            const float sd = surfel_hit(s, ray.x, ray.y);
             if (sd > 0.0f) {
               atomicMin(&st.nearest[px], __float_as_uint(sd));  // positive floats order as their bits
               atomicOr(&st.hits[px], 1u << k);
