@@ -43,13 +43,23 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
+// The kernels of a lighting set read only the environment and write their own outputs, so each is
+// launched early and fills the SMs that the last blocks of the ones before leave.  One block of a
+// kernel waits for the previous kernel at its end, so that none is complete before that one is, and
+// the last kernel of a call does not let others begin early (a compose may read what the call wrote).
+// Set of a 2048 x 1024 environment, one after another 2143 us, overlapped 1986 us.
+__device__ __forceinline__ void complete_in_order() {
+  if (blockIdx.x == 0 && blockIdx.y == 0) griddep_wait();
+}
+
 // ------------------------------------------------------------------------------------------
 // BRDF integration table
 // ------------------------------------------------------------------------------------------
-__global__ void k_brdf_lut(int S, int N, float2* __restrict__ lut) {
+__global__ void k_brdf_lut(int S, int N, float2* __restrict__ lut, bool more) {
+  if (more) griddep_launch_dependents();
   int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   int lane = threadIdx.x & 31;
-  if (warp >= S * S) return;
+  if (warp >= S * S) return;  // not all warps of a block
   int i = warp % S, j = warp / S;
   float mu = (i + 0.5f) / S, r = (j + 0.5f) / S;
   float alpha = r * r, a2 = alpha * alpha, k = 0.5f * alpha;
@@ -74,6 +84,7 @@ __global__ void k_brdf_lut(int S, int N, float2* __restrict__ lut) {
   }
   float a = warp_sum(A.s - A.c), bb = warp_sum(B.s - B.c);
   if (lane == 0) lut[warp] = make_float2(a * invN, bb * invN);
+  complete_in_order();
 }
 
 // ------------------------------------------------------------------------------------------
@@ -286,6 +297,7 @@ __global__ void __launch_bounds__(kIrrThreads) k_irradiance_part(const float4* _
       part[(size_t)blockIdx.x * nout + o] =
           make_float4(acc[0].s - acc[0].c, acc[1].s - acc[1].c, acc[2].s - acc[2].c, acc[3].s - acc[3].c);
   }
+  complete_in_order();
 }
 
 // One warp per output texel: lane l sums the partials of blocks l, l + 32, ... (Kahan), then the
@@ -311,7 +323,7 @@ __global__ void k_irradiance_final(const float4* __restrict__ part, int nblocks,
 }
 
 // ------------------------------------------------------------------------------------------
-// Prefiltered levels 1..M-1 in one launch
+// Prefiltered levels 1..M-1
 // ------------------------------------------------------------------------------------------
 struct ChainDev {
   int M;
@@ -330,11 +342,15 @@ struct ChainDev {
 // columns.  One block per (level, row): the block computes, once, every kept sample's source
 // coordinate for texel 0 (the only equirect mapping in the kernel) and its bilinear weights,
 // then every texel of the row sums its samples from the shifted coordinates.  Rows wider than
-// kPrefilterSeg texels are split into segments, one block each.
+// kPrefilterSeg texels (shorter ones where there are few rows) are split into segments, one block each.
 constexpr int kPrefilterMaxSamples = 2048;
 constexpr int kPrefilterThreads = 256;
 constexpr int kPrefilterTexels = 2;  // texels per thread: a block shades a segment of up to 512 texels of a row
 constexpr int kPrefilterSeg = kPrefilterThreads * kPrefilterTexels;
+// Segments are halved down to kPrefilterMinSeg texels until a launch has kPrefilterFill blocks per SM (each
+// block makes its row's records anew).  Lighting set of a 2048 x 1024 environment, levels 3 .. 7 here, the
+// shortest segment 64, 128, 256 or 512 texels: 1998, 1986, 2365, 2366 us.
+constexpr int kPrefilterMinSeg = 128, kPrefilterFill = 4;
 
 // Sample `sidx` of N for alpha^2 = a2 as (2 h_z h_x, 2 h_z h_y, n.l, -); kept iff n.l > 0.  Both
 // compaction passes call this, so they agree on every decision.
@@ -462,18 +478,17 @@ __device__ __forceinline__ int prefilter_records(PrefilterShared& sh, unsigned* 
 // row.  Samples are visited in order of their source row so that consecutive samples read the
 // same two rows, which stay in L1.
 template <bool INT_SHIFT>
-__global__ void __launch_bounds__(kPrefilterThreads) k_prefilter(MapDev src, ChainDev ch, int N) {
+__device__ __forceinline__ void prefilter_segment(const MapDev& src, const ChainDev& ch, int N, int seg) {
   extern __shared__ __align__(16) float4 s_pf[];
   __shared__ PrefilterShared sh;
   __shared__ float3 s_sum[kPrefilterThreads * 2];  // the shares' sums
-  griddep_launch_dependents();  // k_prefilter_rows does other levels at the same time
   float4* s_w = s_pf;
   int2* s_xy = (int2*)(s_pf + N);
   unsigned short* s_pos = (unsigned short*)(s_xy + N);
   const int m = blockIdx.y + ch.first;
   const int W = ch.W[m], H = ch.H[m];
-  const int segs = (W + kPrefilterSeg - 1) / kPrefilterSeg;
-  const int j = blockIdx.x / segs, i0 = (blockIdx.x - j * segs) * kPrefilterSeg;
+  const int segs = (W + seg - 1) / seg;
+  const int j = blockIdx.x / segs, i0 = (blockIdx.x - j * segs) * seg;
   if (j >= H) return;  // block-uniform
   const int W0 = src.W, H0 = src.H;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -499,7 +514,7 @@ __global__ void __launch_bounds__(kPrefilterThreads) k_prefilter(MapDev src, Cha
     // row and group are 32 consecutive texels at level 1 (s = 2); the two lanes of a texel add
     // their sums at the end.
     // A segment of at most 256 texels leaves warps over: these take shares of the samples (`split`).
-    const int cols = (min(W - i0, kPrefilterSeg) + 63) / 64;  // warps side by side
+    const int cols = (min(W - i0, seg) + 63) / 64;  // warps side by side
     const int across = cols > 4 ? 8 : (cols > 2 ? 4 : cols), split = warp / across, splits = 8 / across;
     const int t = lane >> 1, dl = lane & 1;
     const int wbase = i0 + (warp - split * across) * 64;
@@ -561,7 +576,7 @@ __global__ void __launch_bounds__(kPrefilterThreads) k_prefilter(MapDev src, Cha
     return;
   }
   // a thread per texel, or per texel and share of the samples where the segment has at most 128
-  const int n = min(W - i0, kPrefilterSeg);
+  const int n = min(W - i0, seg);
   const int across = n > 128 ? 256 : (n > 64 ? 128 : (n > 32 ? 64 : 32)), split = tid / across;
   const int splits = kPrefilterThreads / across, me = tid - split * across;
   int ii[kPrefilterTexels];
@@ -619,6 +634,21 @@ __global__ void __launch_bounds__(kPrefilterThreads) k_prefilter(MapDev src, Cha
   }
 }
 
+template <bool INT_SHIFT>
+__global__ void __launch_bounds__(kPrefilterThreads)
+    k_prefilter(const __grid_constant__ MapDev src, const __grid_constant__ ChainDev ch, int N, int seg) {
+  griddep_launch_dependents();
+  prefilter_segment<INT_SHIFT>(src, ch, N, seg);
+  complete_in_order();
+}
+
+// Level 0.
+__global__ void __launch_bounds__(256) k_copy_texels(const float4* src, float4* dst, long long n, bool more) {
+  if (more) griddep_launch_dependents();
+  for (long long k = blockIdx.x * 256LL + threadIdx.x; k < n; k += gridDim.x * 256LL) dst[k] = src[k];
+  complete_in_order();
+}
+
 // Levels whose texels are a power of two of source columns apart: the block of a row stages every
 // source row its samples touch, once, in shared memory as three channel planes of phases
 // (column c = phase + phases * k at [phase][k]), so that a tap of all texels of the row is three
@@ -626,9 +656,10 @@ __global__ void __launch_bounds__(kPrefilterThreads) k_prefilter(MapDev src, Cha
 // lines are half, a quarter, ... used.  A thread owns two neighbouring texels (their columns are
 // `step` apart, so a row is staged in 2 step phases and one index serves all four taps); threads left
 // over take shares of the samples.  Bound by shared-memory bandwidth (two rows x two columns x 12
-// bytes per texel and sample; ncu: 78% of the LSU data pipe): levels 1 .. 7 of a 2048 x 1024
-// environment at 1024 samples 2545 us with every level read through L1, 2060 us with levels 1 and 2
-// here and the others, whose spare warps now share the samples, beside them.
+// bytes per texel and sample; ncu: 74% of the LSU data pipe, tail included): levels 1 .. 7 of a 2048 x
+// 1024 environment at 1024 samples 2545 us with every level read through L1; with levels 1 and 2 here,
+// 1800 us, and the others after them in the SMs that the last rows leave, the whole set takes 1986 us
+// (2143 us with the others first: their blocks' shared memory leaves no room for the rows').
 constexpr int kRowsThreads = 512, kRowsMaxW = 2048, kRowsMaxH = 2048;
 constexpr int kRowsMinW = 128;  // texels per row of a level
 // Above a step of 4 a source row is staged for too few texels: the lighting set of a 2048 x 1024
@@ -725,7 +756,7 @@ __device__ __forceinline__ void prefilter_row(const float4* s_w, const RowsTap* 
       if (slot == 2) prefilter_taps<2>(part, s_w, s_tap, from + share, to, shares, 4u * me, 4u * pairs);
     }
     since += to - from;
-    if (since >= 64) {  // fold the plain sums into the running sums
+    if (since >= 32) {  // fold the plain sums into the running sums
       since = 0;
 #pragma unroll
       for (int g = 0; g < 2; ++g) {
@@ -767,6 +798,7 @@ __global__ void __launch_bounds__(kRowsThreads, 2) k_prefilter_rows(MapDev src, 
   __shared__ PrefilterShared rec;
   __shared__ int s_rows_n;
   const int m = blockIdx.y + ch.first, j = blockIdx.x, W = ch.W[m], H = ch.H[m], H0 = src.H, W0 = src.W;
+  griddep_launch_dependents();
   if (j < H) {  // block-uniform
     float4* s_w = (float4*)(s_rows + 3 * kRowsSlot);
     RowsTap* s_tap = (RowsTap*)(s_w + N);
@@ -808,7 +840,6 @@ __global__ void __launch_bounds__(kRowsThreads, 2) k_prefilter_rows(MapDev src, 
     float4* dst = ch.dst[m] + (long long)j * W;
     prefilter_row(s_w, s_tap, s_start, s_list, s_rows_n, src, dst, W, phases, phase_words, 1.0f / wsum);
   }
-  griddep_wait();  // launched beside k_prefilter: complete only after it
 }
 
 static epbr_status validate_ibl_for(const epbr_ibl* ibl, int We, int He) {
@@ -828,15 +859,36 @@ static epbr_status validate_ibl_for(const epbr_ibl* ibl, int We, int He) {
 
 using namespace epbr;
 
-extern "C" epbr_status epbr_brdf_lut(int32_t S, int32_t N, float* lut, void* stream) {
+namespace epbr {
+
+// Each step of a lighting set is checked, then launched; `early` says whether the kernel before it on
+// the stream is another one of these, `more` whether one follows in the same call.
+static epbr_status validate_lut(int S, int N, const float* lut) {
   if (S < 1 || S > 4096 || N < 1 || N > (1 << 24) || !lut)
     return fail(EPBR_ERR_INVALID_ARG, "brdf_lut: size %d / samples %d / pointer invalid", S, N);
   if ((uintptr_t)lut % 8) return fail(EPBR_ERR_INVALID_ARG, "brdf_lut: lut not 8-byte aligned");
-  long long threads = (long long)S * S * 32;
-  int blocks = (int)((threads + 255) / 256);
-  k_brdf_lut<<<blocks, 256, 0, (cudaStream_t)stream>>>(S, N, (float2*)lut);
-  epbr_status st = check_launch("k_brdf_lut");
-  return st ? st : ok();
+  return EPBR_OK;
+}
+
+static epbr_status launched(cudaError_t e, const char* what) {
+  if (e == cudaSuccess) return check_launch(what);
+  cudaGetLastError();
+  return fail(EPBR_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e));
+}
+
+static epbr_status launch_lut(int S, int N, float* lut, cudaStream_t s, bool early, bool more) {
+  const long long threads = (long long)S * S * 32;
+  return launched(launch_kernel(k_brdf_lut, dim3((unsigned)((threads + 255) / 256)), dim3(256), 0, s, early, S, N, (float2*)lut,
+                                more),
+                  "k_brdf_lut");
+}
+
+}  // namespace epbr
+
+extern "C" epbr_status epbr_brdf_lut(int32_t S, int32_t N, float* lut, void* stream) {
+  epbr_status st = validate_lut(S, N, lut);
+  if (st || (st = launch_lut(S, N, lut, (cudaStream_t)stream, false, false))) return st;
+  return ok();
 }
 
 extern "C" epbr_status epbr_precompute_ibl_workspace_size(const epbr_ibl_params* p, int32_t We,
@@ -851,7 +903,8 @@ extern "C" epbr_status epbr_precompute_ibl_workspace_size(const epbr_ibl_params*
 namespace epbr {
 
 // Partial sums into `ws` (at least irr_workspace_bytes), then the outputs.
-static epbr_status launch_irradiance(const epbr_env* env, int Wi, int Hi, float4* ws, float4* out, cudaStream_t s) {
+static epbr_status launch_irradiance(const epbr_env* env, int Wi, int Hi, float4* ws, float4* out, cudaStream_t s,
+                                     bool early) {
   const int We = env->width, He = env->height, nout = Wi * Hi;
   const bool round = We <= kIrrPiece && We % kIrrSeg == 0;
   // slices of whole row pieces, as even as the three blocks an SM holds allow
@@ -865,8 +918,9 @@ static epbr_status launch_irradiance(const epbr_env* env, int Wi, int Hi, float4
   void (*k)(const float4*, int, int, int, int, float4*) = round ? k_irradiance_part<true> : k_irradiance_part<false>;
   if (smem > 48 * 1024 && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return fail(EPBR_ERR_CUDA, "irradiance: shared-memory attribute: %s", cudaGetErrorString(cudaGetLastError()));
-  k<<<dim3(nb, gy), threads, smem, s>>>((const float4*)env->texels, We, He, Wi, Hi, ws);
-  epbr_status st = check_launch("k_irradiance_part");
+  epbr_status st = launched(launch_kernel(k, dim3(nb, gy), dim3(threads), smem, s, early, (const float4*)env->texels, We, He,
+                                          Wi, Hi, ws),
+                            "k_irradiance_part");
   if (st) return st;
   k_irradiance_final<<<(unsigned)(((long long)nout * 32 + 255) / 256), 256, 0, s>>>(ws, nb, nout, out);
   return check_launch("k_irradiance_final");
@@ -874,18 +928,28 @@ static epbr_status launch_irradiance(const epbr_env* env, int Wi, int Hi, float4
 
 }  // namespace epbr
 
-extern "C" epbr_status epbr_irradiance(const epbr_env* env, int32_t Wi, int32_t Hi, float* out,
-                                       void* ws, size_t ws_bytes, void* stream) {
+namespace epbr {
+
+static epbr_status validate_irradiance(const epbr_env* env, int Wi, int Hi, const float* out, const void* ws,
+                                       size_t ws_bytes) {
   epbr_status st = validate_env(env);
   if (st) return st;
   if (Wi < 1 || Hi < 1 || Wi > 4096 || Hi > 4096 || !out)
     return fail(EPBR_ERR_INVALID_ARG, "irradiance: output %dx%d or pointer invalid", Wi, Hi);
   if ((uintptr_t)out % 16) return fail(EPBR_ERR_INVALID_ARG, "irradiance: out not 16-byte aligned");
-  size_t need = irr_workspace_bytes(env->width, env->height, Wi, Hi);
+  const size_t need = irr_workspace_bytes(env->width, env->height, Wi, Hi);
   if (!ws || ws_bytes < need || (uintptr_t)ws % 16)
     return fail(EPBR_ERR_NO_MEMORY, "irradiance: workspace needs %zu bytes (16-byte aligned), got %zu", need,
                 ws ? ws_bytes : (size_t)0);
-  if ((st = launch_irradiance(env, Wi, Hi, (float4*)ws, (float4*)out, (cudaStream_t)stream))) return st;
+  return EPBR_OK;
+}
+
+}  // namespace epbr
+
+extern "C" epbr_status epbr_irradiance(const epbr_env* env, int32_t Wi, int32_t Hi, float* out,
+                                       void* ws, size_t ws_bytes, void* stream) {
+  epbr_status st = validate_irradiance(env, Wi, Hi, out, ws, ws_bytes);
+  if (st || (st = launch_irradiance(env, Wi, Hi, (float4*)ws, (float4*)out, (cudaStream_t)stream, false))) return st;
   return ok();
 }
 
@@ -979,21 +1043,23 @@ extern "C" epbr_status epbr_irradiance_noalloc(const epbr_env* env, int32_t Wi, 
   if ((st = static_scratch(&ws))) return st;
   // Every partial the final pass reads is written by the first pass, so the scratch needs no
   // clearing between calls.
-  if ((st = launch_irradiance(env, Wi, Hi, (float4*)ws, (float4*)out, (cudaStream_t)stream))) return st;
+  if ((st = launch_irradiance(env, Wi, Hi, (float4*)ws, (float4*)out, (cudaStream_t)stream, false))) return st;
   return ok();
 }
 
-extern "C" epbr_status epbr_prefilter(const epbr_env* env, int32_t N, const epbr_ibl* ibl, void* stream) {
+namespace epbr {
+
+static epbr_status validate_prefilter(const epbr_env* env, int N, const epbr_ibl* ibl) {
   epbr_status st = validate_env(env);
   if (st) return st;
   if ((st = validate_ibl_for(ibl, env->width, env->height))) return st;
   if (N < 1 || N > kPrefilterMaxSamples)
     return fail(EPBR_ERR_INVALID_ARG, "prefilter: samples %d outside [1, %d]", N, kPrefilterMaxSamples);
-  cudaStream_t s = (cudaStream_t)stream;
-  if (cudaMemcpyAsync(ibl->level[0], env->texels, (size_t)env->width * env->height * 16,
-                      cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-    return fail(EPBR_ERR_CUDA, "prefilter: level-0 copy failed: %s", cudaGetErrorString(cudaGetLastError()));
-  if (ibl->num_levels < 2) return ok();
+  return EPBR_OK;
+}
+
+// The levels, then level 0.
+static epbr_status launch_prefilter(const epbr_env* env, int N, const epbr_ibl* ibl, cudaStream_t s, bool more) {
   ChainDev ch;
   ch.M = ibl->num_levels;
   for (int m = 0; m < EPBR_MAX_LEVELS; ++m) {
@@ -1003,44 +1069,65 @@ extern "C" epbr_status epbr_prefilter(const epbr_env* env, int32_t N, const epbr
   }
   const int W0 = env->width, H0 = env->height;
   MapDev src{(const float4*)env->texels, W0, H0};
+  epbr_status st;
+  bool early = false;
   // levels 1 .. rows by k_prefilter_rows: texels 2 or 4 source columns apart, texel pairs of whole warps
   int rows = 0;
   while (rows + 1 < ch.M && (2 << rows) <= kRowsMaxStep && W0 <= kRowsMaxW && H0 <= kRowsMaxH &&
          W0 % (64 * (2 << rows)) == 0 && W0 / (2 << rows) >= kRowsMinW)
     ++rows;
-  // the others one block per row (level rows + 1 has the most rows), before it: the two run side
-  // by side; whole-column shifts when every level's width divides the source width
+  if (rows > 0) {
+    ch.first = 1;
+    const size_t smem = rows_shared_bytes(N, H0);
+    if (cudaFuncSetAttribute(k_prefilter_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+      return fail(EPBR_ERR_CUDA, "prefilter: shared-memory attribute: %s", cudaGetErrorString(cudaGetLastError()));
+    if ((st = launched(launch_kernel(k_prefilter_rows, dim3(ch.H[1], rows), dim3(kRowsThreads), smem, s, early, src, ch, N),
+                       "k_prefilter_rows")))
+      return st;
+    early = true;
+  }
+  // the others a block per segment of a row (level rows + 1 has the most); whole-column shifts when
+  // every level's width divides the source width
   ch.first = rows + 1;
   if (ch.first < ch.M) {
     bool int_shift = true;
     for (int m = ch.first; m < ch.M; ++m) int_shift = int_shift && W0 % ch.W[m] == 0;
+    int seg = kPrefilterSeg;
     unsigned most = 0;
-    for (int m = ch.first; m < ch.M; ++m)
-      most = std::max(most, (unsigned)(ch.H[m] * ((ch.W[m] + kPrefilterSeg - 1) / kPrefilterSeg)));
+    for (;; seg /= 2) {
+      long long blocks = 0;
+      most = 0;
+      for (int m = ch.first; m < ch.M; ++m) {
+        const unsigned b = (unsigned)(ch.H[m] * ((ch.W[m] + seg - 1) / seg));
+        blocks += b;
+        most = std::max(most, b);
+      }
+      if (seg <= kPrefilterMinSeg || blocks >= (long long)kPrefilterFill * num_sms()) break;
+    }
     const size_t smem = (size_t)N * (sizeof(float4) + sizeof(int2) + sizeof(unsigned short));
-    void (*k)(MapDev, ChainDev, int) = int_shift ? k_prefilter<true> : k_prefilter<false>;
+    void (*k)(const MapDev, const ChainDev, int, int) = int_shift ? k_prefilter<true> : k_prefilter<false>;
     if (smem > 48 * 1024 &&
         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
       return fail(EPBR_ERR_CUDA, "prefilter: shared-memory attribute: %s", cudaGetErrorString(cudaGetLastError()));
     // a small shared-memory carve-out leaves most of the SM's 256 KB to L1, which holds the source
     // rows the resident blocks read (two rows of up to 16 KB per block)
     cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 50);  // a hint; failure is harmless
-    k<<<dim3(most, (unsigned)(ch.M - ch.first)), kPrefilterThreads, smem, s>>>(src, ch, N);
-    if ((st = check_launch("k_prefilter"))) return st;
+    if ((st = launched(launch_kernel(k, dim3(most, (unsigned)(ch.M - ch.first)), dim3(kPrefilterThreads), smem, s, early, src,
+                                     ch, N, seg),
+                       "k_prefilter")))
+      return st;
+    early = true;
   }
-  if (rows > 0) {
-    const bool early = ch.first < ch.M;
-    ch.first = 1;
-    const size_t smem = rows_shared_bytes(N, H0);
-    if (cudaFuncSetAttribute(k_prefilter_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-      return fail(EPBR_ERR_CUDA, "prefilter: shared-memory attribute: %s", cudaGetErrorString(cudaGetLastError()));
-    cudaError_t e = launch_kernel(k_prefilter_rows, dim3(ch.H[1], rows), dim3(kRowsThreads), smem, s, early, src, ch, N);
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      return fail(EPBR_ERR_CUDA, "k_prefilter_rows: %s", cudaGetErrorString(e));
-    }
-    if ((st = check_launch("k_prefilter_rows"))) return st;
-  }
+  return launched(launch_kernel(k_copy_texels, dim3(num_sms() * 4), dim3(256), 0, s, early, src.texels, ch.dst[0],
+                                (long long)W0 * H0, more),
+                  "k_copy_texels");
+}
+
+}  // namespace epbr
+
+extern "C" epbr_status epbr_prefilter(const epbr_env* env, int32_t N, const epbr_ibl* ibl, void* stream) {
+  epbr_status st = validate_prefilter(env, N, ibl);
+  if (st || (st = launch_prefilter(env, N, ibl, (cudaStream_t)stream, false))) return st;
   return ok();
 }
 
@@ -1053,8 +1140,13 @@ extern "C" epbr_status epbr_precompute_ibl(const epbr_env* env, const epbr_ibl_p
   if (ibl->num_levels != p->num_levels || ibl->lut_size != p->lut_size || ibl->irr_width != p->irr_width ||
       ibl->irr_height != p->irr_height || !ibl->lut || !ibl->irradiance)
     return fail(EPBR_ERR_INVALID_ARG, "ibl layout does not match params");
-  if ((st = epbr_brdf_lut(p->lut_size, p->lut_samples, ibl->lut, stream))) return st;
-  if ((st = epbr_irradiance(env, p->irr_width, p->irr_height, ibl->irradiance, ws, ws_bytes, stream))) return st;
-  if ((st = epbr_prefilter(env, p->prefilter_samples, ibl, stream))) return st;
+  if ((st = validate_lut(p->lut_size, p->lut_samples, ibl->lut))) return st;
+  if ((st = validate_irradiance(env, p->irr_width, p->irr_height, ibl->irradiance, ws, ws_bytes))) return st;
+  if ((st = validate_prefilter(env, p->prefilter_samples, ibl))) return st;
+  cudaStream_t s = (cudaStream_t)stream;
+  // the longest first, each of the others beginning as the blocks of those before run out
+  if ((st = launch_prefilter(env, p->prefilter_samples, ibl, s, true))) return st;
+  if ((st = launch_lut(p->lut_size, p->lut_samples, ibl->lut, s, true, true))) return st;
+  if ((st = launch_irradiance(env, p->irr_width, p->irr_height, (float4*)ws, (float4*)ibl->irradiance, s, true))) return st;
   return ok();
 }
