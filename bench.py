@@ -154,11 +154,11 @@ FLOP_SHADOW = 40         # lit pair with shadows: light-view transform (18), 1/z
                          # threshold (2), nine depth compares, the visibility scale (3)
 SHADOW = {"size": 512, "fov_deg": 90.0, "bias_const": 0.02, "bias_slope": 0.01}
 MESH = {"n_lat": 16, "n_lon": 32, "ground_cells": 64, "near": 0.05}
-RASTER_LAUNCHES = 7  # key reset, set-up, three scan kernels, coverage, resolve
-SHADOW_MAP_LAUNCHES = 6  # per group of up to 8 lights: set-up, three scan kernels, coverage, depth resolve
-SHADOW_MAP_GROUP = 8     # (the key reset is a memset)
+RASTER_LAUNCHES = 3  # triangles, queued boxes, resolve (the key reset is a memset)
+SHADOW_MAP_LAUNCHES = 2  # per group of lights, after one fill: triangles, queued boxes
+SHADOW_MAP_GROUP = 9     # lights that the workspace of this mesh and map size has room for
 SURFELS = {"per_sphere": 4000, "ground": 400000, "overlap": 1.2, "seed": 11, "near": 0.05, "tolerance": 0.01}
-SURFEL_LAUNCHES = 10  # depth and sum resets, pixel rays, set-up, three scan kernels, two coverage passes, resolve
+SURFEL_LAUNCHES = 4  # count, list ranges, fill, tiles (the count reset is a memset)
 
 
 def compose_flops(sc, g, n_lights) -> tuple[float, dict]:
@@ -585,7 +585,7 @@ def run_gpu(args):
         compose(gb, shp, hdr, ldr, lights, record)
 
     launches_per_step = 3 + (BLOOM_LAUNCHES if args.bloom else 0) + (RASTER_LAUNCHES if args.mesh else 0) + \
-        (SURFEL_LAUNCHES if args.surfels else 0) + (SHADOW_MAP_LAUNCHES * -(-len(scams) // SHADOW_MAP_GROUP) if smaps_dev else 0)
+        (SURFEL_LAUNCHES if args.surfels else 0) + (1 + SHADOW_MAP_LAUNCHES * -(-len(scams) // SHADOW_MAP_GROUP) if smaps_dev else 0)
     with torch.cuda.stream(stream):
         for _ in range(max(3, args.warmup)):
             step()
@@ -784,7 +784,7 @@ def run_gpu(args):
     if smaps_dev:
         line["shadow_maps"] = {"ms": statistics.mean(a.elapsed_time(b) for a, b in ev_smaps), "maps": len(scams),
                                "size": SHADOW["size"], "triangles": smesh.struct.num_triangles,
-                               "launches": SHADOW_MAP_LAUNCHES * -(-len(scams) // SHADOW_MAP_GROUP)}
+                               "launches": 1 + SHADOW_MAP_LAUNCHES * -(-len(scams) // SHADOW_MAP_GROUP)}
     if args.surfels:
         line["surfels"] = {"ms": statistics.mean(a.elapsed_time(b) for a, b in ev_raster), "surfels": len(srec),
                            "launches": SURFEL_LAUNCHES, **SURFELS}
@@ -913,7 +913,7 @@ def run_edl(args):
                                    f"layers), eye-dome lighting {EDL} with the tone map fused",
                        "l2": "flushed between timed steps (256 MB write)",
                        "parallelism": "independent views per GPU (no collective)"},
-            "roofline": {"bound": "hbm", "kernel": "k_edl (+ fused tone map)", "achieved": nbytes / (edl_ms * 1e-3) / 1e9,
+            "roofline": {"bound": "hbm", "kernel": "k_edl_ring (+ fused tone map)", "achieved": nbytes / (edl_ms * 1e-3) / 1e9,
                          "peak": HBM_PEAK_GBS, "unit": "GB/s",
                          "frac": nbytes / (edl_ms * 1e-3) / 1e9 / HBM_PEAK_GBS, "traffic": None,
                          "algorithmic_bytes": nbytes},

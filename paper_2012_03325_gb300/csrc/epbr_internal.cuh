@@ -18,11 +18,6 @@ epbr_status ok();
 epbr_status check_launch(const char* what);
 int num_sms();
 
-// Exclusive int64 prefix sum of data[0 .. n) in place (raster.cu); sums needs
-// scan_num_blocks(n) + 1 entries and receives the total at sums[scan_num_blocks(n)].
-long long scan_num_blocks(long long n);
-void launch_exclusive_scan(long long* data, long long n, long long* sums, cudaStream_t s);
-
 // Launches kernel k; with `early` under programmatic stream serialisation, so that its blocks may
 // start once every block of the previous kernel on the stream has started and called
 // griddep_launch_dependents (or exited), instead of after that kernel has finished.  A kernel

@@ -23,8 +23,6 @@
 
 namespace epbr {
 
-constexpr int kScanThreads = 256, kScanItems = 4, kScanBlock = kScanThreads * kScanItems;
-
 // 64 bytes, two 32-byte sectors for the coverage's read of a triangle
 struct TriSetup {
   int4 qab;    // snapped screen positions of a and b (1/256 px)
@@ -318,7 +316,7 @@ template <int DEPTH>
 __global__ void __launch_bounds__(256, 3) k_raster_large(const TriSetup* __restrict__ setup, RasterQueue queue, int T, int W,
                                                       long long view_px, void* __restrict__ img) {
   griddep_wait();  // launched early: the queue is complete when k_raster_tri has finished
-  griddep_launch_dependents();
+  if (!DEPTH) griddep_launch_dependents();  // the resolve; the maps' last kernel lets nothing begin early
   const int lane = threadIdx.x & 31;
   const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -353,91 +351,6 @@ __global__ void __launch_bounds__(256, 3) k_raster_large(const TriSetup* __restr
     if (k + warps < singles) next_idx = (unsigned)__ldcg(one - (k + warps)), next = setup[next_idx];
     raster_task<DEPTH>(s, idx, 0, box_width(s) * box_height(s), lane, (unsigned)T, W, view_px, img);
   }
-}
-
-// ---- exclusive int64 scan ------------------------------------------------------------------
-__device__ __forceinline__ long long warp_incl_scan(long long v) {
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    long long n = __shfl_up_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) >= o) v += n;
-  }
-  return v;
-}
-
-// Scans kScanBlock values per block in place (exclusive) and writes the block total.
-__global__ void __launch_bounds__(kScanThreads) k_scan_block(long long* __restrict__ data, long long n,
-                                                             long long* __restrict__ block_sums) {
-  __shared__ long long s_warp[kScanThreads / 32];
-  const long long base = (long long)blockIdx.x * kScanBlock + (long long)threadIdx.x * kScanItems;
-  long long v[kScanItems], run = 0;
-#pragma unroll
-  for (int k = 0; k < kScanItems; ++k) {
-    v[k] = base + k < n ? data[base + k] : 0;
-    run += v[k];
-  }
-  long long incl = warp_incl_scan(run);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 31) s_warp[warp] = incl;
-  __syncthreads();
-  if (warp == 0) {
-    long long w = lane < kScanThreads / 32 ? s_warp[lane] : 0;
-    w = warp_incl_scan(w);
-    if (lane < kScanThreads / 32) s_warp[lane] = w;
-  }
-  __syncthreads();
-  long long prefix = incl - run + (warp > 0 ? s_warp[warp - 1] : 0);
-#pragma unroll
-  for (int k = 0; k < kScanItems; ++k) {
-    if (base + k < n) data[base + k] = prefix;
-    prefix += v[k];
-  }
-  if (threadIdx.x == kScanThreads - 1) block_sums[blockIdx.x] = prefix;
-}
-
-// One block: exclusive scan of the block totals in place; total at sums[nb].
-__global__ void __launch_bounds__(kScanThreads) k_scan_sums(long long* __restrict__ sums, int nb) {
-  __shared__ long long s_warp[kScanThreads / 32];
-  __shared__ long long s_carry;
-  if (threadIdx.x == 0) s_carry = 0;
-  __syncthreads();
-  for (int b0 = 0; b0 < nb; b0 += kScanThreads) {
-    int i = b0 + threadIdx.x;
-    long long v = i < nb ? sums[i] : 0;
-    long long incl = warp_incl_scan(v);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 31) s_warp[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-      long long w = lane < kScanThreads / 32 ? s_warp[lane] : 0;
-      w = warp_incl_scan(w);
-      if (lane < kScanThreads / 32) s_warp[lane] = w;
-    }
-    __syncthreads();
-    long long excl = s_carry + incl - v + (warp > 0 ? s_warp[warp - 1] : 0);
-    if (i < nb) sums[i] = excl;
-    __syncthreads();
-    if (threadIdx.x == kScanThreads - 1) s_carry = excl + v;
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) sums[nb] = s_carry;
-}
-
-__global__ void __launch_bounds__(kScanThreads) k_scan_add(long long* __restrict__ data, long long n,
-                                                           const long long* __restrict__ sums) {
-  const long long base = (long long)blockIdx.x * kScanBlock;
-  const long long add = sums[blockIdx.x];
-  for (int k = threadIdx.x; k < kScanBlock; k += kScanThreads)
-    if (base + k < n) data[base + k] += add;
-}
-
-long long scan_num_blocks(long long n) { return (n + kScanBlock - 1) / kScanBlock; }
-
-void launch_exclusive_scan(long long* data, long long n, long long* sums, cudaStream_t s) {
-  const long long nb = scan_num_blocks(n);
-  k_scan_block<<<(unsigned)nb, kScanThreads, 0, s>>>(data, n, sums);
-  k_scan_sums<<<1, kScanThreads, 0, s>>>(sums, (int)nb);
-  k_scan_add<<<(unsigned)nb, kScanThreads, 0, s>>>(data, n, sums);
 }
 
 // ---- resolve ---------------------------------------------------------------------------------
@@ -515,7 +428,7 @@ struct RasterLayout {
 static RasterLayout raster_layout(long long T, int W, int H, int views = 1) {
   RasterLayout l;
   const long long n = T * views;
-  const size_t count_bytes = align256(sizeof(long long) * (size_t)(scan_num_blocks(n) + 1));
+  const size_t count_bytes = align256(sizeof(long long) * (size_t)((n + 1023) / 1024 + 1));
   l.count = 0;  // followed by the keys: one memset resets both
   l.keys = sizeof(unsigned long long) * kCounters;
   l.setup = align256(l.keys + sizeof(unsigned long long) * (size_t)W * H * views);
