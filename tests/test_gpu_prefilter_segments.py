@@ -44,3 +44,21 @@ def test_set_equals_parts(We, He, M):
     for m in range(M):
         assert torch.equal(a.level(m), b.level(m)), m
     assert torch.equal(a.irradiance().view(4, 8, 4), irr) and torch.equal(a.lut().view(16, 16, 2), lut)
+
+
+@pytest.mark.parametrize("We,He,M", [(64, 32, 1), (512, 256, 6), (750, 31, 5)])
+def test_set_under_capture(We, He, M):
+    env = torch.from_numpy(synth.make_env(10, We, He)).cuda()
+    p = ep.ibl_params(M, 64, 16, 64, 8, 4)
+    a, b = ep.Ibl(p, We, He), ep.Ibl(p, We, He)
+    ep.epbr_precompute_ibl(env, a)
+    ws = torch.empty(ep.epbr_precompute_ibl_workspace_size(p, We, He) + 512, dtype=torch.uint8, device="cuda")
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        ep.epbr_precompute_ibl(env, b, workspace=ws)
+    for _ in range(2):
+        g.replay()
+    torch.cuda.synchronize()
+    for m in range(M):
+        assert torch.equal(a.level(m), b.level(m)), m
+    assert torch.equal(a.irradiance(), b.irradiance()) and torch.equal(a.lut(), b.lut())
