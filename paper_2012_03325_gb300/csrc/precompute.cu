@@ -1106,8 +1106,8 @@ static epbr_status launch_prefilter(const epbr_env* env, int N, const epbr_ibl* 
     }
     const size_t smem = (size_t)N * (sizeof(float4) + sizeof(int2) + sizeof(unsigned short));
     void (*k)(const MapDev, const ChainDev, int, int) = int_shift ? k_prefilter<true> : k_prefilter<false>;
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    // for every count: without it the 48 KB limit also covers the kernel's static 6.3 KB
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
       return fail(EPBR_ERR_CUDA, "prefilter: shared-memory attribute: %s", cudaGetErrorString(cudaGetLastError()));
     // a small shared-memory carve-out leaves most of the SM's 256 KB to L1, which holds the source
     // rows the resident blocks read (two rows of up to 16 KB per block)
