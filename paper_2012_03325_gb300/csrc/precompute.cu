@@ -876,6 +876,16 @@ static epbr_status launched(cudaError_t e, const char* what) {
   return fail(EPBR_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
+// Raises kernel k's limit of dynamic shared memory to `most` bytes, the most that any call needs and
+// never one call's own need: the limit belongs to the function, so a smaller value set by another
+// thread between this thread's setting and its launch would refuse the launch.
+template <typename K>
+static epbr_status allow_shared(K* k, size_t most, const char* what) {
+  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) != cudaSuccess)
+    return fail(EPBR_ERR_CUDA, "%s: shared-memory attribute: %s", what, cudaGetErrorString(cudaGetLastError()));
+  return EPBR_OK;
+}
+
 static epbr_status launch_lut(int S, int N, float* lut, cudaStream_t s, bool early, bool more) {
   const long long threads = (long long)S * S * 32;
   return launched(launch_kernel(k_brdf_lut, dim3((unsigned)((threads + 255) / 256)), dim3(256), 0, s, early, S, N, (float2*)lut,
@@ -915,13 +925,13 @@ static epbr_status launch_irradiance(const epbr_env* env, int Wi, int Hi, float4
   const int threads = nb >= num_sms() ? kIrrThreads : 128, passes = (nout + threads - 1) / threads;
   const int gy = (int)std::min<long long>(std::min(passes, 65535), std::max<long long>(1, room / nb));
   const size_t smem = irr_shared(nullptr, std::min(We, kIrrPiece)).bytes;
+  epbr_status st;
   void (*k)(const float4*, int, int, int, int, float4*) = round ? k_irradiance_part<true> : k_irradiance_part<false>;
-  if (smem > 48 * 1024 && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return fail(EPBR_ERR_CUDA, "irradiance: shared-memory attribute: %s", cudaGetErrorString(cudaGetLastError()));
-  epbr_status st = launched(launch_kernel(k, dim3(nb, gy), dim3(threads), smem, s, early, (const float4*)env->texels, We, He,
-                                          Wi, Hi, ws),
-                            "k_irradiance_part");
-  if (st) return st;
+  if ((st = allow_shared(k, irr_shared(nullptr, kIrrPiece).bytes, "irradiance"))) return st;
+  if ((st = launched(launch_kernel(k, dim3(nb, gy), dim3(threads), smem, s, early, (const float4*)env->texels, We, He, Wi, Hi,
+                                   ws),
+                     "k_irradiance_part")))
+    return st;
   k_irradiance_final<<<(unsigned)(((long long)nout * 32 + 255) / 256), 256, 0, s>>>(ws, nb, nout, out);
   return check_launch("k_irradiance_final");
 }
@@ -1079,8 +1089,7 @@ static epbr_status launch_prefilter(const epbr_env* env, int N, const epbr_ibl* 
   if (rows > 0) {
     ch.first = 1;
     const size_t smem = rows_shared_bytes(N, H0);
-    if (cudaFuncSetAttribute(k_prefilter_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-      return fail(EPBR_ERR_CUDA, "prefilter: shared-memory attribute: %s", cudaGetErrorString(cudaGetLastError()));
+    if ((st = allow_shared(k_prefilter_rows, rows_shared_bytes(kPrefilterMaxSamples, kRowsMaxH), "prefilter"))) return st;
     if ((st = launched(launch_kernel(k_prefilter_rows, dim3(ch.H[1], rows), dim3(kRowsThreads), smem, s, early, src, ch, N),
                        "k_prefilter_rows")))
       return st;
@@ -1104,11 +1113,11 @@ static epbr_status launch_prefilter(const epbr_env* env, int N, const epbr_ibl* 
       }
       if (seg <= kPrefilterMinSeg || blocks >= (long long)kPrefilterFill * num_sms()) break;
     }
-    const size_t smem = (size_t)N * (sizeof(float4) + sizeof(int2) + sizeof(unsigned short));
+    constexpr size_t kSampleBytes = sizeof(float4) + sizeof(int2) + sizeof(unsigned short);
+    const size_t smem = (size_t)N * kSampleBytes;
     void (*k)(const MapDev, const ChainDev, int, int) = int_shift ? k_prefilter<true> : k_prefilter<false>;
     // for every count: without it the 48 KB limit also covers the kernel's static 6.3 KB
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-      return fail(EPBR_ERR_CUDA, "prefilter: shared-memory attribute: %s", cudaGetErrorString(cudaGetLastError()));
+    if ((st = allow_shared(k, kPrefilterMaxSamples * kSampleBytes, "prefilter"))) return st;
     // a small shared-memory carve-out leaves most of the SM's 256 KB to L1, which holds the source
     // rows the resident blocks read (two rows of up to 16 KB per block)
     cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 50);  // a hint; failure is harmless
