@@ -158,7 +158,7 @@ RASTER_LAUNCHES = 3  # triangles, queued boxes, resolve (the key reset is a mems
 SHADOW_MAP_LAUNCHES = 2  # per group of lights, after one fill: triangles, queued boxes
 SHADOW_MAP_GROUP = 9     # lights that the workspace of this mesh and map size has room for
 SURFELS = {"per_sphere": 4000, "ground": 400000, "overlap": 1.2, "seed": 11, "near": 0.05, "tolerance": 0.01}
-SURFEL_LAUNCHES = 4  # count, list ranges, fill, tiles (the count reset is a memset)
+SURFEL_LAUNCHES = 5  # count, list ranges, fill, tiles, heavy tiles (the count reset is a memset)
 
 
 def compose_flops(sc, g, n_lights) -> tuple[float, dict]:
