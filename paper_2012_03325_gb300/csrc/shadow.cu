@@ -1,7 +1,7 @@
 // Shadow maps with 3x3 percentage-closer filtering for the point lights (Sec. 5.1; Williams
 // 1978, Reeves et al. 1987), evaluated inside the compose's light loop.
-//   k_shade_shadow  one pixel per thread in 32x4 blocks, lights and their shadow cameras staged
-//                   in shared memory in chunks of 128; per light (monochrome lights two at a time in
+//   k_shade_shadow  one pixel per thread in 32x4 or 32x8 blocks, lights and their shadow cameras staged
+//                   in shared memory in chunks of 128; per light (longer lists two lights at a time in
 //                   packed FP32x2 arithmetic, the same bits) the direct terms of Eq. 1 and,
 //                   when the light reaches the pixel (n.l > 0), its PCF visibility: the fragment
 //                   projected into the light's map and the 3x3 block of depths around its texel
@@ -13,6 +13,12 @@
 namespace epbr {
 
 constexpr int kShadowChunk = 128;
+// Lists of at least this many lights go two lights at a time, shorter ones (and the diffuse-only mode) one,
+// with more warps for the work per pixel: below, the wider kernel's gain per light does not make up for
+// its 37% of the warps against 50%.  1080p, 512^2 maps, us one / two at a time: 1 light 67 / 74, 4 lights
+// 90 / 94, 8 123 / 125, 12 154 / 155, 16 183 / 182, 24 244 / 242, 64 573 / 551; coloured 67 / 74, 90 / 96,
+// 123 / 127, 154 / 158, 184 / 186, 248 / 248, 581 / 568.
+constexpr int kShadowPairs = 16;
 
 struct ShadowDev {
   const float* maps;
@@ -111,19 +117,19 @@ __device__ __forceinline__ float2 shadow_visibility2(const CamPair& c, const flo
   return make_float2(shadow_visibility(cams, P, map0, S, b0, b1), shadow_visibility(cams + 4, P, map1, S, b0, b1));
 }
 
-// 128 threads, six blocks per SM (80 registers, no spill).  Bound by issue and the LSU data pipe (ncu: 68%
-// and 59%; 459 M warp instructions, 565 M with one light at a time): 1080p with 64 lights and 512^2 maps
-// 577 us one light at a time, 547 us two at a time; 256 threads at 64 (spills), 80 and 96 registers
-// 552, 561 and 680 us, and the taps requested before the light terms 589 us at best.
-constexpr int kShadowBY = 4, kShadowThreads = 32 * kShadowBY;
-template <int FMT, int HDR, bool LDR>
-__global__ void __launch_bounds__(kShadowThreads, 6)
+// PAIRS: 128 threads, six blocks per SM (80 registers); else 256 threads, four blocks (64 registers).  Bound by
+// issue and the LSU data pipe.  Two lights at a time in 256 threads at 64 (spills), 80 and 96 registers took
+// 552, 561 and 680 us against 547 us (1080p, 64 lights, 512^2 maps), the taps requested before the light terms
+// 589 us at best.
+template <int FMT, int HDR, bool LDR, bool PAIRS>
+__global__ void __launch_bounds__(32 * (PAIRS ? 4 : 8), PAIRS ? 6 : 4)
     k_shade_shadow(GbufDev g, CamDev cam, const float4* __restrict__ lights, int NL, IblDev ibl, ShadeDev p,
                    ShadowDev sh, void* hdr, long long hdr_pitch, uint8_t* ldr, long long ldr_pitch) {
   __shared__ float4 s_lights[2 * kShadowChunk];
   __shared__ float4 s_cams[4 * kShadowChunk];
-  __shared__ float4 s_pos[kShadowChunk];  // per light pair (x, x, y, y), (z, z, Ic, Ic)
-  __shared__ __align__(16) CamPair s_pair[kShadowChunk / 2];
+  __shared__ float4 s_pos[PAIRS ? kShadowChunk : 1];  // per light pair (x, x, y, y), (z, z, Ic, Ic)
+  __shared__ __align__(16) CamPair s_pair[PAIRS ? kShadowChunk / 2 : 1];
+  constexpr int kShadowBY = PAIRS ? 4 : 8, kShadowThreads = 32 * kShadowBY;
   const int tid = threadIdx.y * 32 + threadIdx.x;
   const int by = gridDim.y - 1 - blockIdx.y;  // costliest rows first, as k_shade
   const int x = blockIdx.x * 32 + threadIdx.x, y = by * kShadowBY + threadIdx.y;
@@ -140,7 +146,7 @@ __global__ void __launch_bounds__(kShadowThreads, 6)
     for (int q = tid; q < 4 * cnt; q += kShadowThreads) s_cams[q] = __ldg(sh.cams + 4 * (size_t)base + q);
     // a chunk of monochrome lights keeps one sum per kind (each channel's sum would be the same)
     const bool mono = __syncthreads_and(stage_lights(s_lights, lights, base, cnt, tid, kShadowThreads));
-    if (mono && !diffuse_only) {  // block-uniform
+    if (PAIRS && !diffuse_only) {  // block-uniform
       for (int q = tid; q < cnt / 2; q += kShadowThreads) {
         const float4 a = s_lights[4 * q], b = s_lights[4 * q + 2];
         s_pos[2 * q] = make_float4(a.x, b.x, a.y, b.y);
@@ -163,76 +169,81 @@ __global__ void __launch_bounds__(kShadowThreads, 6)
       __syncthreads();
     }
     if (!active) continue;
-    if (mono && !diffuse_only) {
-      float sa = 0.0f, sb = 0.0f, sbf = 0.0f;
+    if (!diffuse_only) {
+      // every light's terms times its visibility, added by `add(light, a, b, bf)`
       const float* map = sh.maps + (size_t)base * sh.map_texels;
-      Geo2 g;
-      g.nx = dup2(s.n.x), g.ny = dup2(s.n.y), g.nz = dup2(s.n.z);
-      g.mnx = dup2(-s.n.x), g.mny = dup2(-s.n.y), g.mnz = dup2(-s.n.z);
-      g.vx = dup2(s.v.x), g.vy = dup2(s.v.y), g.vz = dup2(s.v.z);
-      g.nva = dup2(d.nva), g.alpha = dup2(d.alpha), g.k = dup2(d.k), g.omk = dup2(d.omk);
-      const float2 mPx = dup2(-s.P.x), mPy = dup2(-s.P.y), mPz = dup2(-s.P.z);
-      int i = 0;
-      for (; i + 1 < cnt; i += 2, map += 2 * sh.map_texels) {  // two lights at a time
-        const float4 u = s_pos[i], z = s_pos[i + 1];
-        Terms2 t = light_terms2(g, padd(make_float2(u.x, u.y), mPx), padd(make_float2(u.z, u.w), mPy),
-                                padd(make_float2(z.x, z.y), mPz));
-        // the visibility (1 or less, finite) leaves the zero terms of an unlit light as they are
-        if (t.a.x > 0.0f || t.b.x > 0.0f || t.a.y > 0.0f || t.b.y > 0.0f) {
-          const float2 v = shadow_visibility2(s_pair[i >> 1], s_cams + 4 * i, s.P, mPx, mPy, mPz, map,
-                                              map + sh.map_texels, sh.S, sh.b0, sh.b1);
-          t.a = pmul(t.a, v);
-          t.b = pmul(t.b, v);
-          t.bf = pmul(t.bf, v);
+      auto each = [&](auto add) {
+        int i = 0;
+        if (PAIRS) {
+          Geo2 g;
+          g.nx = dup2(s.n.x), g.ny = dup2(s.n.y), g.nz = dup2(s.n.z);
+          g.mnx = dup2(-s.n.x), g.mny = dup2(-s.n.y), g.mnz = dup2(-s.n.z);
+          g.vx = dup2(s.v.x), g.vy = dup2(s.v.y), g.vz = dup2(s.v.z);
+          g.nva = dup2(d.nva), g.alpha = dup2(d.alpha), g.k = dup2(d.k), g.omk = dup2(d.omk);
+          const float2 mPx = dup2(-s.P.x), mPy = dup2(-s.P.y), mPz = dup2(-s.P.z);
+          for (; i + 1 < cnt; i += 2, map += 2 * sh.map_texels) {  // two lights at a time
+            const float4 u = s_pos[i], z = s_pos[i + 1];
+            Terms2 t = light_terms2(g, padd(make_float2(u.x, u.y), mPx), padd(make_float2(u.z, u.w), mPy),
+                                    padd(make_float2(z.x, z.y), mPz));
+            // the visibility (1 or less, finite) leaves the zero terms of an unlit light as they are
+            if (t.a.x > 0.0f || t.b.x > 0.0f || t.a.y > 0.0f || t.b.y > 0.0f) {
+              const float2 v = shadow_visibility2(s_pair[i >> 1], s_cams + 4 * i, s.P, mPx, mPy, mPz, map,
+                                                  map + sh.map_texels, sh.S, sh.b0, sh.b1);
+              t.a = pmul(t.a, v);
+              t.b = pmul(t.b, v);
+              t.bf = pmul(t.bf, v);
+            }
+            add(i, z.z, t.a.x, t.b.x, t.bf.x);
+            add(i + 1, z.w, t.a.y, t.b.y, t.bf.y);
+          }
         }
-        sa = fmaf(z.w, t.a.y, fmaf(z.z, t.a.x, sa));
-        sb = fmaf(z.w, t.b.y, fmaf(z.z, t.b.x, sb));
-        sbf = fmaf(z.w, t.bf.y, fmaf(z.z, t.bf.x, sbf));
-      }
-      for (; i < cnt; ++i, map += sh.map_texels) {
-        const float4 lp = s_lights[2 * i];
-        LightTerms t = light_terms(s, d, lp);
-        if (t.a > 0.0f || t.b > 0.0f) {
-          const float v = shadow_visibility(s_cams + 4 * i, s.P, map, sh.S, sh.b0, sh.b1);
-          t.a *= v;
-          t.b *= v;
-          t.bf *= v;
+        for (; i < cnt; ++i, map += sh.map_texels) {
+          const float4 lp = s_lights[2 * i];
+          LightTerms t = light_terms(s, d, lp);
+          if (t.a > 0.0f || t.b > 0.0f) {
+            const float v = shadow_visibility(s_cams + 4 * i, s.P, map, sh.S, sh.b0, sh.b1);
+            t.a *= v;
+            t.b *= v;
+            t.bf *= v;
+          }
+          add(i, lp.w, t.a, t.b, t.bf);
         }
-        sa = sa + lp.w * t.a;  // lp.w: the light's Ic
-        sb = sb + lp.w * t.b;
-        sbf = sbf + lp.w * t.bf;
+      };
+      if (mono) {
+        float sa = 0.0f, sb = 0.0f, sbf = 0.0f;
+        each([&](int, float Ic, float a, float b, float bf) {
+          sa = fmaf(Ic, a, sa);
+          sb = fmaf(Ic, b, sb);
+          sbf = fmaf(Ic, bf, sbf);
+        });
+        d.sa = d.sa + f3(sa, sa, sa);
+        d.sb = d.sb + f3(sb, sb, sb);
+        d.sbf = d.sbf + f3(sbf, sbf, sbf);
+      } else {
+        float3 sa = d.sa, sb = d.sb, sbf = d.sbf;
+        each([&](int i, float, float a, float b, float bf) {
+          const float3 lc = xyz(s_lights[2 * i + 1]);
+          sa = sa + lc * a;
+          sb = sb + lc * b;
+          sbf = sbf + lc * bf;
+        });
+        d.sa = sa;
+        d.sb = sb;
+        d.sbf = sbf;
       }
-      d.sa = d.sa + f3(sa, sa, sa);
-      d.sb = d.sb + f3(sb, sb, sb);
-      d.sbf = d.sbf + f3(sbf, sbf, sbf);
       continue;
     }
-    float3 sa = d.sa, sb = d.sb, sbf = d.sbf;
+    float3 sa = d.sa;
     for (int i = 0; i < cnt; ++i) {
       float4 lp = s_lights[2 * i], lc = s_lights[2 * i + 1];
       const float* map = sh.maps + (size_t)(base + i) * sh.map_texels;
-      if (diffuse_only) {
-        float3 L = xyz(lp) - s.P;
-        float rs = rsqrt_ftz(fmaf(L.x, L.x, fmaf(L.y, L.y, fmaf(L.z, L.z, 1e-30f))));
-        float w = rs * rs * fmaxf(dot3(s.n, L) * rs, 0.0f);
-        if (w > 0.0f) w *= shadow_visibility(s_cams + 4 * i, s.P, map, sh.S, sh.b0, sh.b1);
-        sa = sa + xyz(lc) * w;
-        continue;
-      }
-      LightTerms t = light_terms(s, d, lp);
-      if (t.a > 0.0f || t.b > 0.0f) {
-        float v = shadow_visibility(s_cams + 4 * i, s.P, map, sh.S, sh.b0, sh.b1);
-        t.a *= v;
-        t.b *= v;
-        t.bf *= v;
-      }
-      sa = sa + xyz(lc) * t.a;
-      sb = sb + xyz(lc) * t.b;
-      sbf = sbf + xyz(lc) * t.bf;
+      float3 L = xyz(lp) - s.P;
+      float rs = rsqrt_ftz(fmaf(L.x, L.x, fmaf(L.y, L.y, fmaf(L.z, L.z, 1e-30f))));
+      float w = rs * rs * fmaxf(dot3(s.n, L) * rs, 0.0f);
+      if (w > 0.0f) w *= shadow_visibility(s_cams + 4 * i, s.P, map, sh.S, sh.b0, sh.b1);
+      sa = sa + xyz(lc) * w;
     }
     d.sa = sa;
-    d.sb = sb;
-    d.sbf = sbf;
   }
   if (!inside) return;
   if (active && NL > 0) {
@@ -251,12 +262,16 @@ __global__ void __launch_bounds__(kShadowThreads, 6)
 }
 
 template <int FMT, int HDR>
-static cudaError_t launch_shadow(dim3 grd, dim3 blk, cudaStream_t st, const GbufDev& g, const CamDev& c,
-                                 const float4* L, int NL, const IblDev& ibl, const ShadeDev& p, const ShadowDev& sh,
-                                 void* hdr, long long hp, uint8_t* ldr, long long lp) {
+static cudaError_t launch_shadow(cudaStream_t st, const GbufDev& g, const CamDev& c, const float4* L, int NL,
+                                 const IblDev& ibl, const ShadeDev& p, const ShadowDev& sh, void* hdr, long long hp,
+                                 uint8_t* ldr, long long lp) {
   const bool early = (p.flags & EPBR_SHADE_EARLY_START) != 0;
-  cudaError_t e = launch_kernel(ldr ? k_shade_shadow<FMT, HDR, true> : k_shade_shadow<FMT, HDR, false>, grd, blk, 0, st,
-                                early, g, c, L, NL, ibl, p, sh, hdr, hp, ldr, lp);
+  const bool pairs = NL >= kShadowPairs && !(p.flags & EPBR_SHADE_DIFFUSE_ONLY);
+  const int by = pairs ? 4 : 8;
+  auto k = pairs ? (ldr ? k_shade_shadow<FMT, HDR, true, true> : k_shade_shadow<FMT, HDR, false, true>)
+                 : (ldr ? k_shade_shadow<FMT, HDR, true, false> : k_shade_shadow<FMT, HDR, false, false>);
+  cudaError_t e = launch_kernel(k, dim3((g.W + 31) / 32, (g.H + by - 1) / by), dim3(32, by), 0, st, early, g, c, L, NL, ibl,
+                                p, sh, hdr, hp, ldr, lp);
   if (e != cudaSuccess) cudaGetLastError();
   return e;
 }
@@ -272,20 +287,17 @@ epbr_status launch_shade_shadows(const GbufDev& g, const CamDev& c, int fmt, con
                 "negative / non-finite bias");
   ShadowDev sh{s->maps, (const float4*)s->cameras, (long long)s->size * s->size, s->size, s->bias_const,
                s->bias_slope};
-  dim3 blk(32, kShadowBY), grd((g.W + 31) / 32, (g.H + kShadowBY - 1) / kShadowBY);
   cudaError_t e;
   if (fmt == EPBR_GBUFFER_FP32) {
     if (hdr_format == EPBR_HDR_RGBA32F)
-      e = launch_shadow<EPBR_GBUFFER_FP32, EPBR_HDR_RGBA32F>(grd, blk, st, g, c, L, NL, ibl, p, sh, hdr, hp, ldr, lp);
+      e = launch_shadow<EPBR_GBUFFER_FP32, EPBR_HDR_RGBA32F>(st, g, c, L, NL, ibl, p, sh, hdr, hp, ldr, lp);
     else
-      e = launch_shadow<EPBR_GBUFFER_FP32, EPBR_HDR_RGBA16F>(grd, blk, st, g, c, L, NL, ibl, p, sh, hdr, hp, ldr, lp);
+      e = launch_shadow<EPBR_GBUFFER_FP32, EPBR_HDR_RGBA16F>(st, g, c, L, NL, ibl, p, sh, hdr, hp, ldr, lp);
   } else {
     if (hdr_format == EPBR_HDR_RGBA32F)
-      e = launch_shadow<EPBR_GBUFFER_COMPACT, EPBR_HDR_RGBA32F>(grd, blk, st, g, c, L, NL, ibl, p, sh, hdr, hp, ldr,
-                                                                lp);
+      e = launch_shadow<EPBR_GBUFFER_COMPACT, EPBR_HDR_RGBA32F>(st, g, c, L, NL, ibl, p, sh, hdr, hp, ldr, lp);
     else
-      e = launch_shadow<EPBR_GBUFFER_COMPACT, EPBR_HDR_RGBA16F>(grd, blk, st, g, c, L, NL, ibl, p, sh, hdr, hp, ldr,
-                                                                lp);
+      e = launch_shadow<EPBR_GBUFFER_COMPACT, EPBR_HDR_RGBA16F>(st, g, c, L, NL, ibl, p, sh, hdr, hp, ldr, lp);
   }
   if (e != cudaSuccess) return fail(EPBR_ERR_CUDA, "k_shade_shadow: %s", cudaGetErrorString(e));
   return check_launch("k_shade_shadow");
