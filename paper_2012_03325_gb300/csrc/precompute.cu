@@ -5,14 +5,13 @@
 //                       sums of 64 and 8 texels and single texels at its ends (Kahan across pieces)
 //   k_irradiance_final  one warp per output: lanes sum the block partials, a shuffle butterfly
 //                       adds the lanes (fixed order: deterministic), then the ratio
-//   k_prefilter_rows    GGX-prefiltered levels 1 and 2 of the usual maps, one block per row of a level:
-//                       the row's sample geometry computed once (the sampling frame turns with the
-//                       texel about the pole axis), each texel sums its samples at shifted columns of
-//                       source rows staged in shared memory
-//   k_prefilter         the other levels, source rows read through L1
+//   k_prefilter         GGX-prefiltered levels 1..M-1, a block per segment of a row of a level: the
+//                       row's sample geometry computed once (the sampling frame turns with the texel
+//                       about the pole axis), each texel sums its samples at shifted columns
 #include <cuda.h>  // CUcontext and CUresult for the context queries (fetched at run time)
 
 #include <algorithm>
+#include <type_traits>
 #include <mutex>
 
 #include "epbr_internal.cuh"
@@ -334,7 +333,6 @@ __global__ void k_irradiance_final(const float4* __restrict__ part, int nblocks,
 // ------------------------------------------------------------------------------------------
 struct ChainDev {
   int M;
-  int first;  // the first level a launch writes
   int W[EPBR_MAX_LEVELS], H[EPBR_MAX_LEVELS];
   float4* dst[EPBR_MAX_LEVELS];
 };
@@ -355,9 +353,11 @@ constexpr int kPrefilterThreads = 256;
 constexpr int kPrefilterTexels = 2;  // texels per thread: a block shades a segment of up to 512 texels of a row
 constexpr int kPrefilterSeg = kPrefilterThreads * kPrefilterTexels;
 // Segments are halved down to kPrefilterMinSeg texels until a launch has kPrefilterFill blocks per SM (each
-// block makes its row's records anew).  Lighting set of a 2048 x 1024 environment, levels 3 .. 7 here, the
-// shortest segment 64, 128, 256 or 512 texels: 1998, 1986, 2365, 2366 us.
-constexpr int kPrefilterMinSeg = 128, kPrefilterFill = 4;
+// block makes its row's records anew).  Prefilter (us) with the shortest segment 64, 128, 256 or 512 texels: 2048 x
+// 64, 8 levels, 1024 samples 224, 252, 357, 315; 512 x 256, 6 levels, 512 samples 121, 103, 98, 98; 2048 x 1024
+// 2083 with each.  With 2, 3, 4 or 8 blocks per SM: 1024 x 512, 8 levels, 1024 samples 524, 524, 566, 654; 750 x
+// 375, 6 levels, 512 samples 384, 356, 356, 357.
+constexpr int kPrefilterMinSeg = 128, kPrefilterFill = 3;
 
 // Sample `sidx` of N for alpha^2 = a2 as (2 h_z h_x, 2 h_z h_y, n.l, -); kept iff n.l > 0.  Both
 // compaction passes call this, so they agree on every decision.
@@ -381,24 +381,24 @@ __device__ __forceinline__ float2 prefilter_src_xy(float3 l, int W0, int H0) {
 // positions; the sort keys (N unsigned) occupy the weights' space until the records are written.
 struct PrefilterShared {
   int base[kPrefilterMaxSamples / 32 + 1];
-  float wsum[16];
+  float wsum[kPrefilterThreads / 32];
 };
 
 // The samples of row j of level m as records in order of source row (a deterministic bitonic sort of
-// (source row + 1, sample) keys), by a block of THREADS threads.  `keyed(keys, ns)` sees the sorted
-// keys, `emit(position, sample (.z = n.l), source x, y for texel 0)` writes a record.  Returns the
-// number of kept samples and their weight sum sum_k n.l_k (the same for every texel of the level).
-template <int THREADS, typename Keyed, typename Emit>
+// (source row, sample) keys), by a whole block: `emit(position, sample (.z = n.l), source x, y for texel 0)`
+// writes a record.  Returns the number of kept samples and their weight sum sum_k n.l_k (the same for every
+// texel of the level).
+template <typename Emit>
 __device__ __forceinline__ int prefilter_records(PrefilterShared& sh, unsigned* s_key, unsigned short* s_pos, int m,
                                                  int M, int j, int W, int H, int W0, int H0, int N, float& wsum,
-                                                 Keyed keyed, Emit emit) {
+                                                 Emit emit) {
   const float r = (float)m / (float)(M - 1);
   const float a2 = r * r * r * r;
   const float invN = 1.0f / N;
   const int groups = (N + 31) / 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // kept samples per group of 32, then an exclusive prefix over the groups (sample order)
-  for (int gi = warp; gi < groups; gi += THREADS / 32) {
+  for (int gi = warp; gi < groups; gi += kPrefilterThreads / 32) {
     int sidx = gi * 32 + lane;
     bool keep = sidx < N && prefilter_sample(sidx, a2, invN).z > 0.0f;
     unsigned bal = __ballot_sync(0xffffffffu, keep);
@@ -423,7 +423,7 @@ __device__ __forceinline__ int prefilter_records(PrefilterShared& sh, unsigned* 
   const float3 T = f3(-cp0, 0.0f, -sp0);
   const float3 B = cross3(n, T);
   // pass A: each kept sample's source row, as a sort key
-  for (int gi = warp; gi < groups; gi += THREADS / 32) {
+  for (int gi = warp; gi < groups; gi += kPrefilterThreads / 32) {
     int sidx = gi * 32 + lane;
     float4 e = sidx < N ? prefilter_sample(sidx, a2, invN) : make_float4(0, 0, 0, 0);
     bool keep = sidx < N && e.z > 0.0f;
@@ -431,17 +431,17 @@ __device__ __forceinline__ int prefilter_records(PrefilterShared& sh, unsigned* 
     if (keep) {
       const int q = sh.base[gi] + __popc(bal & ((1u << lane) - 1u));
       const float2 xy = prefilter_src_xy(T * e.x + B * e.y + n * e.z, W0, H0);
-      const int iy = min(max((int)floorf(xy.y), -1), H0 - 1) + 1;
+      const int iy = min(max((int)floorf(xy.y), 0), H0 - 1);
       s_key[q] = ((unsigned)iy << 16) | (unsigned)q;
     }
   }
   int P = 1;
   while (P < ns) P <<= 1;
-  for (int q = ns + tid; q < P; q += THREADS) s_key[q] = 0xffffffffu;
+  for (int q = ns + tid; q < P; q += kPrefilterThreads) s_key[q] = 0xffffffffu;
   __syncthreads();
   for (int k = 2; k <= P; k <<= 1) {
     for (int jj = k >> 1; jj > 0; jj >>= 1) {
-      for (int q = tid; q < P; q += THREADS) {
+      for (int q = tid; q < P; q += kPrefilterThreads) {
         const int o = q ^ jj;
         if (o > q) {
           const unsigned a = s_key[q], b = s_key[o];
@@ -454,12 +454,11 @@ __device__ __forceinline__ int prefilter_records(PrefilterShared& sh, unsigned* 
       __syncthreads();
     }
   }
-  for (int q = tid; q < ns; q += THREADS) s_pos[s_key[q] & 0xffffu] = (unsigned short)q;
-  keyed(s_key, ns);
+  for (int q = tid; q < ns; q += kPrefilterThreads) s_pos[s_key[q] & 0xffffu] = (unsigned short)q;
   __syncthreads();  // the keys are dead from here: their space takes the records
   // pass B: the records at their sorted positions; the weights summed in sample order
   float wpart = 0.0f;
-  for (int gi = warp; gi < groups; gi += THREADS / 32) {
+  for (int gi = warp; gi < groups; gi += kPrefilterThreads / 32) {
     int sidx = gi * 32 + lane;
     float4 e = sidx < N ? prefilter_sample(sidx, a2, invN) : make_float4(0, 0, 0, 0);
     bool keep = sidx < N && e.z > 0.0f;
@@ -475,7 +474,7 @@ __device__ __forceinline__ int prefilter_records(PrefilterShared& sh, unsigned* 
   __syncthreads();
   wsum = 0.0f;
 #pragma unroll
-  for (int w = 0; w < THREADS / 32; ++w) wsum += sh.wsum[w];
+  for (int w = 0; w < kPrefilterThreads / 32; ++w) wsum += sh.wsum[w];
   return ns;
 }
 
@@ -483,7 +482,8 @@ __device__ __forceinline__ int prefilter_records(PrefilterShared& sh, unsigned* 
 // Wm) stores the four bilinear weights times n.l and (column, row); otherwise the two row weights
 // times n.l and the source x coordinate (the column fraction then varies along the row), and the
 // row.  Samples are visited in order of their source row so that consecutive samples read the
-// same two rows, which stay in L1.
+// same two rows, which stay in L1.  A plain FP32 sum takes 64 samples, compensated sums take the
+// plain ones and the shares.
 template <bool INT_SHIFT>
 __device__ __forceinline__ void prefilter_segment(const MapDev& src, const ChainDev& ch, int N, int seg) {
   extern __shared__ __align__(16) float4 s_pf[];
@@ -492,7 +492,7 @@ __device__ __forceinline__ void prefilter_segment(const MapDev& src, const Chain
   float4* s_w = s_pf;
   int2* s_xy = (int2*)(s_pf + N);
   unsigned short* s_pos = (unsigned short*)(s_xy + N);
-  const int m = blockIdx.y + ch.first;
+  const int m = blockIdx.y + 1;
   const int W = ch.W[m], H = ch.H[m];
   const int segs = (W + seg - 1) / seg;
   const int j = blockIdx.x / segs, i0 = (blockIdx.x - j * segs) * seg;
@@ -500,8 +500,8 @@ __device__ __forceinline__ void prefilter_segment(const MapDev& src, const Chain
   const int W0 = src.W, H0 = src.H;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   float wsum;
-  const int ns = prefilter_records<kPrefilterThreads>(
-      sh, (unsigned*)s_pf, s_pos, m, ch.M, j, W, H, W0, H0, N, wsum, [](const unsigned*, int) {},
+  const int ns = prefilter_records(
+      sh, (unsigned*)s_pf, s_pos, m, ch.M, j, W, H, W0, H0, N, wsum,
       [&](int p, float4 e, float2 xy) {
         const float xf = floorf(xy.x), yf = floorf(xy.y);
         const float fx = xy.x - xf, fy = xy.y - yf;
@@ -527,46 +527,59 @@ __device__ __forceinline__ void prefilter_segment(const MapDev& src, const Chain
     const int wbase = i0 + (warp - split * across) * 64;
     int col[4];
     bool ong[4];
-    float3 acc[4], part[4];
+    Kahan3 acc[4];
+    float3 part[4];
 #pragma unroll
     for (int g = 0; g < 4; ++g) {
       const int i = wbase + 16 * g + t;
       ong[g] = wbase + 16 * g < W;  // warp-uniform: whether group g has texels
       col[g] = min(i, W - 1) * step_i + dl;
-      acc[g] = part[g] = f3(0, 0, 0);
+      part[g] = f3(0, 0, 0);
     }
-    int since = 0;
+    // WHOLE: all samples in turn, the usual case, whose loop a stride known only at run time slows down (1000 x
+    // 500, 3 levels, 128 samples: 121 us instead of 83)
+    auto sum = [&](auto whole) {
+      constexpr bool WHOLE = decltype(whole)::value;
+      int since = 0;
 #pragma unroll 2
-    for (int q = split; q < (ong[0] ? ns : 0); q += splits) {
-      const float4 w = s_w[q];
-      const int2 xy = s_xy[q];
-      const int r0 = max(xy.y, 0) * W0, r1 = min(xy.y + 1, H0 - 1) * W0;
-      const float wa = dl ? w.y : w.x, wb = dl ? w.w : w.z;  // this column's weights in rows r0, r1
-#pragma unroll
-      for (int g = 0; g < 4; ++g) {
-        if (!ong[g]) continue;
-        int c = xy.x + col[g];  // in [-1, 2 W0 - 1)
-        c = c < 0 ? c + W0 : (c >= W0 ? c - W0 : c);
-        const float4 a = __ldg(src.texels + (r0 + c)), p = __ldg(src.texels + (r1 + c));
-        part[g].x = fmaf(wa, a.x, fmaf(wb, p.x, part[g].x));
-        part[g].y = fmaf(wa, a.y, fmaf(wb, p.y, part[g].y));
-        part[g].z = fmaf(wa, a.z, fmaf(wb, p.z, part[g].z));
-      }
-      if ((++since & 63) == 0) {  // fold every 64 samples' plain sums into the running sums
+      for (int q = WHOLE ? 0 : split; q < ns; q += WHOLE ? 1 : splits) {
+        const float4 w = s_w[q];
+        const int2 xy = s_xy[q];
+        const int r0 = max(xy.y, 0) * W0, r1 = min(xy.y + 1, H0 - 1) * W0;
+        const float wa = dl ? w.y : w.x, wb = dl ? w.w : w.z;  // this column's weights in rows r0, r1
 #pragma unroll
         for (int g = 0; g < 4; ++g) {
-          acc[g] = acc[g] + part[g];
-          part[g] = f3(0, 0, 0);
+          if (!ong[g]) continue;
+          int c = xy.x + col[g];  // in [-1, 2 W0 - 1)
+          c = c < 0 ? c + W0 : (c >= W0 ? c - W0 : c);
+          const float4 a = __ldg(src.texels + (r0 + c)), p = __ldg(src.texels + (r1 + c));
+          part[g].x = fmaf(wa, a.x, fmaf(wb, p.x, part[g].x));
+          part[g].y = fmaf(wa, a.y, fmaf(wb, p.y, part[g].y));
+          part[g].z = fmaf(wa, a.z, fmaf(wb, p.z, part[g].z));
+        }
+        if (WHOLE ? (q & 63) == 63 : (++since & 63) == 0) {  // fold every 64 samples' plain sums into the running sums
+#pragma unroll
+          for (int g = 0; g < 4; ++g) {
+            acc[g].add(part[g]);
+            part[g] = f3(0, 0, 0);
+          }
         }
       }
+    };
+    if (splits == 1) {
+      if (!ong[0]) return;  // warp-uniform, after the last barrier
+      sum(std::true_type());
+    } else if (ong[0]) {
+      sum(std::false_type());
     }
 #pragma unroll
     for (int g = 0; g < 4; ++g) {
-      float3 v = acc[g] + part[g];
+      acc[g].add(part[g]);
+      float3 v = acc[g].value();
       v.x += __shfl_xor_sync(0xffffffffu, v.x, 1);
       v.y += __shfl_xor_sync(0xffffffffu, v.y, 1);
       v.z += __shfl_xor_sync(0xffffffffu, v.z, 1);
-      acc[g] = v;
+      part[g] = v;
       if (splits > 1 && dl == 0) s_sum[warp * 64 + 16 * g + t] = v;
     }
     if (splits > 1) __syncthreads();  // block-uniform
@@ -576,7 +589,7 @@ __device__ __forceinline__ void prefilter_segment(const MapDev& src, const Chain
       const int i = wbase + 16 * g + t;
       if (dl || !ong[g] || i >= W) continue;
       Kahan3 v;
-      v.add(acc[g]);
+      v.add(part[g]);
       for (int k = 1; k < splits; ++k) v.add(s_sum[(warp + k * across) * 64 + 16 * g + t]);
       const float3 o = v.value() * inv;
       ch.dst[m][(long long)j * W + i] = make_float4(o.x, o.y, o.z, 1.0f);
@@ -589,44 +602,54 @@ __device__ __forceinline__ void prefilter_segment(const MapDev& src, const Chain
   const int splits = kPrefilterThreads / across, me = tid - split * across;
   int ii[kPrefilterTexels];
   bool on[kPrefilterTexels];  // block-uniform: whether the segment has a texel group c
-  float3 acc[kPrefilterTexels], part[kPrefilterTexels];
+  Kahan3 acc[kPrefilterTexels];
+  float3 part[kPrefilterTexels];
 #pragma unroll
   for (int c = 0; c < kPrefilterTexels; ++c) {
     on[c] = c * kPrefilterThreads < n;
     ii[c] = min(i0 + c * kPrefilterThreads + me, W - 1);  // duplicates of the last texel are not stored
-    acc[c] = part[c] = f3(0, 0, 0);
+    part[c] = f3(0, 0, 0);
   }
-  int since = 0;
+  auto sum = [&](auto whole) {
+    constexpr bool WHOLE = decltype(whole)::value;
+    int since = 0;
 #pragma unroll 2
-  for (int q = split; q < ns; q += splits) {
-    const float4 w = s_w[q];
-    const int2 xy = s_xy[q];
-    const int r0 = max(xy.y, 0) * W0, r1 = min(xy.y + 1, H0 - 1) * W0;
-#pragma unroll
-    for (int c = 0; c < kPrefilterTexels; ++c) {
-      if (!on[c]) continue;
-      const float x = fmaf((float)ii[c], step_f, w.z);
-      const float xf = floorf(x), fx = x - xf;
-      int x0 = (int)xf;
-      const float4 wq = make_float4(w.x * (1.0f - fx), w.x * fx, w.y * (1.0f - fx), w.y * fx);
-      x0 = x0 < 0 ? x0 + W0 : (x0 >= W0 ? x0 - W0 : x0);
-      const int x1 = x0 + 1 == W0 ? 0 : x0 + 1;
-      const float4 a = __ldg(src.texels + (r0 + x0)), b = __ldg(src.texels + (r0 + x1));
-      const float4 p = __ldg(src.texels + (r1 + x0)), d = __ldg(src.texels + (r1 + x1));
-      part[c].x = fmaf(wq.x, a.x, fmaf(wq.y, b.x, fmaf(wq.z, p.x, fmaf(wq.w, d.x, part[c].x))));
-      part[c].y = fmaf(wq.x, a.y, fmaf(wq.y, b.y, fmaf(wq.z, p.y, fmaf(wq.w, d.y, part[c].y))));
-      part[c].z = fmaf(wq.x, a.z, fmaf(wq.y, b.z, fmaf(wq.z, p.z, fmaf(wq.w, d.z, part[c].z))));
-    }
-    if ((++since & 63) == 0) {  // fold every 64 samples' plain sums into the running sums
+    for (int q = WHOLE ? 0 : split; q < ns; q += WHOLE ? 1 : splits) {
+      const float4 w = s_w[q];
+      const int2 xy = s_xy[q];
+      const int r0 = max(xy.y, 0) * W0, r1 = min(xy.y + 1, H0 - 1) * W0;
 #pragma unroll
       for (int c = 0; c < kPrefilterTexels; ++c) {
-        acc[c] = acc[c] + part[c];
-        part[c] = f3(0, 0, 0);
+        if (!on[c]) continue;
+        const float x = fmaf((float)ii[c], step_f, w.z);
+        const float xf = floorf(x), fx = x - xf;
+        int x0 = (int)xf;
+        const float4 wq = make_float4(w.x * (1.0f - fx), w.x * fx, w.y * (1.0f - fx), w.y * fx);
+        x0 = x0 < 0 ? x0 + W0 : (x0 >= W0 ? x0 - W0 : x0);
+        const int x1 = x0 + 1 == W0 ? 0 : x0 + 1;
+        const float4 a = __ldg(src.texels + (r0 + x0)), b = __ldg(src.texels + (r0 + x1));
+        const float4 p = __ldg(src.texels + (r1 + x0)), d = __ldg(src.texels + (r1 + x1));
+        part[c].x = fmaf(wq.x, a.x, fmaf(wq.y, b.x, fmaf(wq.z, p.x, fmaf(wq.w, d.x, part[c].x))));
+        part[c].y = fmaf(wq.x, a.y, fmaf(wq.y, b.y, fmaf(wq.z, p.y, fmaf(wq.w, d.y, part[c].y))));
+        part[c].z = fmaf(wq.x, a.z, fmaf(wq.y, b.z, fmaf(wq.z, p.z, fmaf(wq.w, d.z, part[c].z))));
+      }
+      if (WHOLE ? (q & 63) == 63 : (++since & 63) == 0) {  // fold every 64 samples' plain sums into the running sums
+#pragma unroll
+        for (int c = 0; c < kPrefilterTexels; ++c) {
+          acc[c].add(part[c]);
+          part[c] = f3(0, 0, 0);
+        }
       }
     }
-  }
+  };
+  if (splits == 1)
+    sum(std::true_type());
+  else
+    sum(std::false_type());
   if (splits > 1) {  // block-uniform
-    s_sum[tid] = acc[0] + part[0];
+    acc[0].add(part[0]);
+    part[0] = f3(0, 0, 0);
+    s_sum[tid] = acc[0].value();
     __syncthreads();
     if (split > 0) return;
   }
@@ -634,8 +657,8 @@ __device__ __forceinline__ void prefilter_segment(const MapDev& src, const Chain
   for (int c = 0; c < kPrefilterTexels; ++c) {
     const int i = i0 + c * kPrefilterThreads + me;
     if (on[c] && i < W) {
-      Kahan3 v;
-      v.add(acc[c] + part[c]);
+      Kahan3 v = acc[c];
+      v.add(part[c]);
       for (int k = 1; k < splits; ++k) v.add(s_sum[me + k * across]);
       const float3 o = v.value() * inv;
       ch.dst[m][(long long)j * W + i] = make_float4(o.x, o.y, o.z, 1.0f);
@@ -643,8 +666,13 @@ __device__ __forceinline__ void prefilter_segment(const MapDev& src, const Chain
   }
 }
 
+// Bound by L1 (16 bytes per tap, of which 12 are used) and its latency: two blocks per SM with up to 128 registers,
+// so that the loads of two samples are under way, take 2083 us for the levels of a 2048 x 1024 environment (8
+// levels, 1024 samples), three blocks 2202 us; 1024 x 512, 3 levels, 128 samples 76 and 92 us.  Source rows
+// staged in shared memory for levels 1 and 2 took 2020 us for the first and 229 us for the second: a row is
+// staged for too few samples unless the lobe is narrow and the count high.
 template <bool INT_SHIFT>
-__global__ void __launch_bounds__(kPrefilterThreads)
+__global__ void __launch_bounds__(kPrefilterThreads, 2)
     k_prefilter(const __grid_constant__ MapDev src, const __grid_constant__ ChainDev ch, int N, int seg) {
   griddep_launch_dependents();
   prefilter_segment<INT_SHIFT>(src, ch, N, seg);
@@ -656,221 +684,6 @@ __global__ void __launch_bounds__(256) k_copy_texels(const float4* src, float4* 
   if (more) griddep_launch_dependents();
   for (long long k = blockIdx.x * 256LL + threadIdx.x; k < n; k += gridDim.x * 256LL) dst[k] = src[k];
   complete_in_order();
-}
-
-// Levels whose texels are a power of two of source columns apart: the block of a row stages every
-// source row its samples touch, once, in shared memory as three channel planes of phases
-// (column c = phase + phases * k at [phase][k]), so that a tap of all texels of the row is three
-// conflict-free reads of consecutive words, 12 bytes per texel instead of the 16 of an L1 read whose
-// lines are half, a quarter, ... used.  A thread owns two neighbouring texels (their columns are
-// `step` apart, so a row is staged in 2 step phases and one index serves all four taps); threads left
-// over take shares of the samples.  Bound by shared-memory bandwidth (two rows x two columns x 12
-// bytes per texel and sample; ncu: 74% of the LSU data pipe, tail included): levels 1 .. 7 of a 2048 x
-// 1024 environment at 1024 samples 2545 us with every level read through L1; with levels 1 and 2 here,
-// 1800 us, and the others after them in the SMs that the last rows leave, the whole set takes 1986 us
-// (2143 us with the others first: their blocks' shared memory leaves no room for the rows').
-constexpr int kRowsThreads = 512, kRowsMaxW = 2048, kRowsMaxH = 2048;
-constexpr int kRowsMinW = 128;  // texels per row of a level
-// Above a step of 4 a source row is staged for too few texels: the lighting set of a 2048 x 1024
-// environment takes 2316, 2145 and 2248 us with steps up to 2, 4 and 8.
-constexpr int kRowsMaxStep = 4;
-// A plain FP32 sum takes at most this many samples (four taps each), however many lie between two source
-// rows (1052 of 2048 over a 2048 x 64 environment), before it is added to a compensated running sum: the
-// rounding of the sums is then below that of 64 samples per tap column and plain running sums (k_prefilter),
-// 3.5e-8 against 5.4e-8 rms for 1000 samples (both orders replayed on the host).  Lighting set of a 2048 x 1024 environment, sums of whole
-// rows, plain, 1984 us; of at most 32 samples, plain, 2005; compensated 2028, and 2050 where every row goes
-// through the loop of the long ones.
-constexpr int kRowsFold = 32;
-constexpr int kRowsPlane = kRowsMaxW + 32;     // words per channel: phases padded by 32 / phases words
-constexpr int kRowsSlot = 3 * kRowsPlane;      // words per staged row; three of them: two in use, one being filled
-
-// A sample as the taps read it: byte offset of k for texel 0, then byte offsets of the phases of the
-// two tap columns of an even texel and of the odd texel after it (relative to k, so 4 more where a
-// column belongs to the next k).
-struct RowsTap {
-  unsigned k;
-  unsigned even, odd;  // first column | second column << 16
-  unsigned pad;
-};
-
-__device__ __forceinline__ RowsTap rows_tap(int c, int step, int phases, int phase_words) {
-  const int p = c & (phases - 1);
-  auto at = [&](int d) { return (unsigned)(((p + d) & (phases - 1)) * phase_words + (p + d >= phases ? 1 : 0)) * 4u; };
-  return RowsTap{(unsigned)(c / phases) * 4u, at(0) | (at(1) << 16), at(step) | (at(step + 1) << 16), 0u};
-}
-
-extern __shared__ __align__(16) float s_rows[];
-
-// Adds samples from, from + stride, ... below to, between the rows in slots SLOT and SLOT + 1 (modulo
-// 3), to the texel pair whose even texel is k4 / 4 pairs along the row of n4 / 4 pairs.
-template <int SLOT>
-__device__ __forceinline__ void prefilter_taps(float3 (&part)[2], const float4* s_w, const RowsTap* s_tap, int from,
-                                               int to, int stride, unsigned k4, unsigned n4) {
-  constexpr int kTop = SLOT * kRowsSlot, kBot = (SLOT + 1) % 3 * kRowsSlot;
-  for (int q = from; q < to; q += stride) {
-    const float4 w = s_w[q];
-    const uint4 t = *(const uint4*)(s_tap + q);
-    unsigned k = t.x + k4;
-    k = min(k, k - n4);  // wrapped round the row
-#pragma unroll
-    for (int g = 0; g < 2; ++g) {
-      const unsigned o = g ? t.z : t.y;
-      const float* a = (const float*)((const char*)s_rows + (k + (o & 0xffffu)));
-      const float* b = (const float*)((const char*)s_rows + (k + (o >> 16)));
-      part[g].x = fmaf(w.x, a[kTop], fmaf(w.y, b[kTop], fmaf(w.z, a[kBot], fmaf(w.w, b[kBot], part[g].x))));
-      part[g].y = fmaf(w.x, a[kTop + kRowsPlane], fmaf(w.y, b[kTop + kRowsPlane],
-                  fmaf(w.z, a[kBot + kRowsPlane], fmaf(w.w, b[kBot + kRowsPlane], part[g].y))));
-      part[g].z = fmaf(w.x, a[kTop + 2 * kRowsPlane], fmaf(w.y, b[kTop + 2 * kRowsPlane],
-                  fmaf(w.z, a[kBot + 2 * kRowsPlane], fmaf(w.w, b[kBot + 2 * kRowsPlane], part[g].z))));
-    }
-  }
-}
-
-// s_list: the `rows` source rows that are read (r + 1, -1 and H0 the clamped edges), in ascending
-// order, a sample's two rows next to each other.
-__device__ __forceinline__ void prefilter_row(const float4* s_w, const RowsTap* s_tap, const unsigned short* s_start,
-                                              const unsigned short* s_list, int rows, const MapDev& src,
-                                              float4* __restrict__ dst, int W, int phases, int phase_words, float inv) {
-  const int tid = threadIdx.x, W0 = src.W, H0 = src.H;
-  const int pairs = W / 2, share = tid / pairs, shares = kRowsThreads / pairs, me = tid - share * pairs;
-  constexpr int kLoads = kRowsMaxW / kRowsThreads;
-  float4 v[kLoads];
-  auto load = [&](int k0) {
-    const float4* row = src.texels + (size_t)min(max((int)s_list[k0] - 1, 0), H0 - 1) * W0;
-#pragma unroll
-    for (int k = 0; k < kLoads; ++k)
-      if (tid + k * kRowsThreads < W0) v[k] = __ldg(row + tid + k * kRowsThreads);
-  };
-  const int log2p = 31 - __clz(phases);
-  auto store = [&](int slot) {
-#pragma unroll
-    for (int k = 0; k < kLoads; ++k) {
-      const int c = tid + k * kRowsThreads;
-      if (c >= W0) continue;
-      float* q = s_rows + slot * kRowsSlot + (c & (phases - 1)) * phase_words + (c >> log2p);
-      q[0] = v[k].x, q[kRowsPlane] = v[k].y, q[2 * kRowsPlane] = v[k].z;
-      if (c < phases) {  // each phase's first column once more after its last
-        q += pairs;
-        q[0] = v[k].x, q[kRowsPlane] = v[k].y, q[2 * kRowsPlane] = v[k].z;
-      }
-    }
-  };
-  Kahan3 acc[2];
-  float3 part[2];
-  part[0] = part[1] = f3(0, 0, 0);
-  auto fold = [&]() {  // the plain sums into the running sums
-#pragma unroll
-    for (int g = 0; g < 2; ++g) {
-      acc[g].add(part[g]);
-      part[g] = f3(0, 0, 0);
-    }
-  };
-  load(0);
-  store(0);
-  load(1);
-  store(1);
-  __syncthreads();
-  int since = 0;
-  for (int k = 0, slot = 0; k + 1 < rows; ++k) {
-    if (k + 2 < rows) load(k + 2);
-    const int from = s_start[s_list[k]], to = s_start[s_list[k] + 1];  // the samples between rows k and k + 1
-    if (since + (to - from) > kRowsFold) fold(), since = 0;
-    since += to - from;
-    if (share < shares) {
-      auto taps = [&](int a, int b) {
-        if (slot == 0) prefilter_taps<0>(part, s_w, s_tap, a + share, b, shares, 4u * me, 4u * pairs);
-        if (slot == 1) prefilter_taps<1>(part, s_w, s_tap, a + share, b, shares, 4u * me, 4u * pairs);
-        if (slot == 2) prefilter_taps<2>(part, s_w, s_tap, a + share, b, shares, 4u * me, 4u * pairs);
-      };
-      if (to - from <= kRowsFold) {
-        taps(from, to);
-      } else {
-#pragma unroll 1
-        for (int q = from; q < to; q += kRowsFold) {
-          taps(q, min(to, q + kRowsFold));
-          fold();
-        }
-      }
-    }
-    if (k + 2 < rows) store(slot == 0 ? 2 : slot - 1);  // the slot of row k - 1
-    slot = slot == 2 ? 0 : slot + 1;
-    __syncthreads();
-  }
-  fold();
-  float3 sum[2] = {acc[0].value(), acc[1].value()};
-  if (shares > 1) {  // block-uniform; the staged rows are dead
-    float3* s_sum = (float3*)s_rows;
-    s_sum[2 * tid] = sum[0];
-    s_sum[2 * tid + 1] = sum[1];
-    __syncthreads();
-    if (share == 0) {
-      for (int k = 1; k < shares; ++k) {
-        acc[0].add(s_sum[2 * (tid + k * pairs)]);
-        acc[1].add(s_sum[2 * (tid + k * pairs) + 1]);
-      }
-      sum[0] = acc[0].value(), sum[1] = acc[1].value();
-    }
-  }
-  if (share > 0) return;
-#pragma unroll
-  for (int g = 0; g < 2; ++g) {
-    const float3 o = sum[g] * inv;
-    dst[2 * me + g] = make_float4(o.x, o.y, o.z, 1.0f);
-  }
-}
-
-// Dynamic shared memory: the staged rows, N float4 weights (first the sort keys), N taps, N sorted
-// positions, H0 + 3 first samples (of source row r at [r + 1]), the list of source rows.
-size_t rows_shared_bytes(int N, int H0) {
-  return 4 * (size_t)(3 * kRowsSlot) + (sizeof(float4) + sizeof(RowsTap) + 2) * (size_t)N + 4 * (size_t)(H0 + 3);
-}
-
-__global__ void __launch_bounds__(kRowsThreads, 2) k_prefilter_rows(MapDev src, ChainDev ch, int N) {
-  __shared__ PrefilterShared rec;
-  __shared__ int s_rows_n;
-  const int m = blockIdx.y + ch.first, j = blockIdx.x, W = ch.W[m], H = ch.H[m], H0 = src.H, W0 = src.W;
-  griddep_launch_dependents();
-  if (j < H) {  // block-uniform
-    float4* s_w = (float4*)(s_rows + 3 * kRowsSlot);
-    RowsTap* s_tap = (RowsTap*)(s_w + N);
-    unsigned short* s_pos = (unsigned short*)(s_tap + N);
-    unsigned short* s_start = s_pos + N;
-    unsigned short* s_list = s_start + H0 + 3;
-    const int step = 1 << m, phases = 2 * step, phase_words = (W0 + 32) / phases;
-    float wsum;
-    prefilter_records<kRowsThreads>(
-        rec, (unsigned*)s_w, s_pos, m, ch.M, j, W, H, W0, H0, N, wsum,
-        [&](const unsigned* key, int n) {
-          // start[k] = number of samples whose source row + 1 is below k
-          for (int q = threadIdx.x; q <= n; q += kRowsThreads) {
-            const int lo = q > 0 ? (int)(key[q - 1] >> 16) + 1 : 0, hi = q < n ? (int)(key[q] >> 16) : H0 + 2;
-            for (int k = lo; k <= hi; ++k) s_start[k] = (unsigned short)q;
-          }
-        },
-        [&](int p, float4 e, float2 xy) {
-          const float xf = floorf(xy.x), yf = floorf(xy.y);
-          const float fx = xy.x - xf, fy = xy.y - yf;
-          const float wt = e.z * (1.0f - fy), wb = e.z * fy;
-          s_w[p] = make_float4(wt * (1.0f - fx), wt * fx, wb * (1.0f - fx), wb * fx);
-          const int c = (int)xf;
-          s_tap[p] = rows_tap(c < 0 ? c + W0 : (c >= W0 ? c - W0 : c), step, phases, phase_words);
-        });
-    // the source rows with a sample (between them and the next) and the rows after these
-    if (threadIdx.x < 32) {
-      int n = 0;
-      for (int r0 = 0; r0 < H0 + 2; r0 += 32) {
-        const int r = r0 + threadIdx.x;  // source row + 1
-        const bool need = r < H0 + 2 && s_start[r + 1] > s_start[max(r - 1, 0)];
-        const unsigned bal = __ballot_sync(0xffffffffu, need);
-        if (need) s_list[n + __popc(bal & ((1u << threadIdx.x) - 1u))] = (unsigned short)r;
-        n += __popc(bal);
-      }
-      if (threadIdx.x == 0) s_rows_n = n;
-    }
-    __syncthreads();
-    float4* dst = ch.dst[m] + (long long)j * W;
-    prefilter_row(s_w, s_tap, s_start, s_list, s_rows_n, src, dst, W, phases, phase_words, 1.0f / wsum);
-  }
 }
 
 static epbr_status validate_ibl_for(const epbr_ibl* ibl, int We, int He) {
@@ -1112,32 +925,17 @@ static epbr_status launch_prefilter(const epbr_env* env, int N, const epbr_ibl* 
   MapDev src{(const float4*)env->texels, W0, H0};
   epbr_status st;
   bool early = false;
-  // levels 1 .. rows by k_prefilter_rows: texels 2 or 4 source columns apart, texel pairs of whole warps
-  int rows = 0;
-  while (rows + 1 < ch.M && (2 << rows) <= kRowsMaxStep && W0 <= kRowsMaxW && H0 <= kRowsMaxH &&
-         W0 % (64 * (2 << rows)) == 0 && W0 / (2 << rows) >= kRowsMinW)
-    ++rows;
-  if (rows > 0) {
-    ch.first = 1;
-    const size_t smem = rows_shared_bytes(N, H0);
-    if ((st = allow_shared(k_prefilter_rows, rows_shared_bytes(kPrefilterMaxSamples, kRowsMaxH), "prefilter"))) return st;
-    if ((st = launched(launch_kernel(k_prefilter_rows, dim3(ch.H[1], rows), dim3(kRowsThreads), smem, s, early, src, ch, N),
-                       "k_prefilter_rows")))
-      return st;
-    early = true;
-  }
-  // the others a block per segment of a row (level rows + 1 has the most); whole-column shifts when
-  // every level's width divides the source width
-  ch.first = rows + 1;
-  if (ch.first < ch.M) {
+  // a block per segment of a row (level 1 has the most); whole-column shifts when every level's width
+  // divides the source width
+  if (ch.M > 1) {
     bool int_shift = true;
-    for (int m = ch.first; m < ch.M; ++m) int_shift = int_shift && W0 % ch.W[m] == 0;
+    for (int m = 1; m < ch.M; ++m) int_shift = int_shift && W0 % ch.W[m] == 0;
     int seg = kPrefilterSeg;
     unsigned most = 0;
     for (;; seg /= 2) {
       long long blocks = 0;
       most = 0;
-      for (int m = ch.first; m < ch.M; ++m) {
+      for (int m = 1; m < ch.M; ++m) {
         const unsigned b = (unsigned)(ch.H[m] * ((ch.W[m] + seg - 1) / seg));
         blocks += b;
         most = std::max(most, b);
@@ -1149,10 +947,11 @@ static epbr_status launch_prefilter(const epbr_env* env, int N, const epbr_ibl* 
     void (*k)(const MapDev, const ChainDev, int, int) = int_shift ? k_prefilter<true> : k_prefilter<false>;
     // for every count: without it the 48 KB limit also covers the kernel's static 6.3 KB
     if ((st = allow_shared(k, kPrefilterMaxSamples * kSampleBytes, "prefilter"))) return st;
-    // a small shared-memory carve-out leaves most of the SM's 256 KB to L1, which holds the source
-    // rows the resident blocks read (two rows of up to 16 KB per block)
-    cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 50);  // a hint; failure is harmless
-    if ((st = launched(launch_kernel(k, dim3(most, (unsigned)(ch.M - ch.first)), dim3(kPrefilterThreads), smem, s, early, src,
+    // a small shared-memory carve-out leaves most of the SM's 256 KB to L1, which holds the source rows the
+    // resident blocks read (two rows of up to 16 KB per block); 40% (100 KB) holds two blocks of up to 1600
+    // samples: levels of a 2048 x 1024 environment at 50% 2101 us, at 40% 2060, at 25% (one block) 2321
+    cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 40);  // a hint; failure is harmless
+    if ((st = launched(launch_kernel(k, dim3(most, (unsigned)(ch.M - 1)), dim3(kPrefilterThreads), smem, s, early, src,
                                      ch, N, seg),
                        "k_prefilter")))
       return st;

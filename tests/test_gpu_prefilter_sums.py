@@ -1,9 +1,9 @@
 """Rounding of the prefiltered levels' sums, over environments of one colour: every texel's weighted mean is
 that colour, whatever the geometry, so what is left is the rounding of the sums.  With u = 2^-24: a plain
-sum of 32 samples (128 FMAs) has a rounding error of about u sqrt(128 / 9) = 3.8 u of itself, independent
-between sums, 0.5 u of the whole for 64 of them; the compensated sums over them, the weights' sum, its
-reciprocal and the product add at most 1.5 u.  Bound: 1.5 u + 6 x 0.5 u = 4.5 u.  (One plain sum over the
-1052 samples that fall between two rows of the first environment has about 11 u.)"""
+sum of 128 FMAs has a rounding error of about u sqrt(128 / 9) = 3.8 u of itself, independent between sums,
+0.5 u of the whole for 64 of them; the compensated sums over them, the weights' sum, its reciprocal and
+the product add at most 1.5 u.  Bound: 1.5 u + 6 x 0.5 u = 4.5 u.  (A plain sum over the 1052 samples
+that fall between two rows of the first environment has about 11 u.)"""
 import numpy as np
 import pytest
 
@@ -25,7 +25,7 @@ def test_one_colour(We, He, M):
     env[..., :3] = torch.from_numpy(colour).cuda()
     ibl = ep.Ibl(ep.ibl_params(M, N, 8, 8, 4, 2), We, He)
     ep.epbr_prefilter(env, N, ibl)
-    for m in (1, 2):  # rows staged in shared memory
+    for m in (1, 2):
         if We >> m < 128:
             continue
         g = ibl.level(m).cpu().numpy()[..., :3].astype(np.float64)
