@@ -3,6 +3,8 @@
 //   k_irradiance_part   exact-quadrature irradiance, per-block partial sums over a slice of source
 //                       row pieces: a row's hemisphere is one interval of columns, summed from
 //                       sums of 64 and 8 texels and single texels at its ends (Kahan across pieces)
+//   k_irradiance_texels the same for narrow environments, every output and texel (packed FP32x2 over
+//                       output pairs, plain sums per staged tile, Kahan across tiles)
 //   k_irradiance_final  one warp per output: lanes sum the block partials, a shuffle butterfly
 //                       adds the lanes (fixed order: deterministic), then the ratio
 //   k_prefilter         GGX-prefiltered levels 1..M-1, a block per segment of a row of a level: the
@@ -168,8 +170,8 @@ __host__ __device__ inline IrrShared irr_shared(char* base, int n) {
   return s;
 }
 
-// Bound by issue (the terms of every output and row): 39 us for a 2048 x 1024 environment, 319 us
-// when every output summed every source texel in packed FP32x2 arithmetic (62% of the FMA pipe).
+// Bound by issue (the terms of every output and row): 39 us for a 2048 x 1024 environment, 319 us by
+// k_irradiance_texels.
 // Each block takes the row pieces of its slice, a thread one output per pass (blockIdx.y and its
 // stride: the passes).  A piece's sums (L w and w, with the row's solid angle) are added to the
 // slice totals with Kahan compensation.  ROUND: a piece is a whole row of whole segments, so the
@@ -302,6 +304,97 @@ __global__ void __launch_bounds__(kIrrThreads) k_irradiance_part(const float4* _
     if (o < nout)
       part[(size_t)blockIdx.x * nout + o] =
           make_float4(acc[0].s - acc[0].c, acc[1].s - acc[1].c, acc[2].s - acc[2].c, acc[3].s - acc[3].c);
+  }
+  complete_in_order();
+}
+
+// Rows of fewer columns than this, unless of whole segments.  32 x 16 outputs by texels / by intervals (us): 16 x 8
+// environment 12 / 26, 40 x 20 31 / 66, 64 x 32 37 / 33 (whole segments), 96 x 50 36 / 45, 130 x 65 35 / 39, 250 x 125
+// 37 / 27, 37 x 4001 38 / 193.
+constexpr int kIrrNarrow = 192;
+constexpr int kIrrTexThreads = 128;
+constexpr int kIrrOutPerThread = 4;  // outputs per thread and pass (two packed pairs): 512 per pass
+constexpr int kIrrTile = 256;        // source texels staged per step
+
+// Narrow environments, whose rows have too few columns for sums of 8 and 64: each block sums over its slice
+// of source texels, a thread owns kIrrOutPerThread outputs of a group of 512 (blockIdx.y and its stride) as
+// two pairs whose arithmetic runs in packed FP32x2 instructions.
+// A source texel is staged once per tile as d Omega (max(n.d, 0) Omega = max(n.(d Omega), 0) since
+// Omega > 0) and L, every value duplicated into both halves of a pair: (dx, dx, dy, dy),
+// (dz, dz, Lr, Lr), (Lg, Lg, Lb, Lb).  Per tile the four sums of each output (L w and w) are
+// plain FP32; the tile's sums are then added to the slice totals with Kahan compensation.
+__global__ void __launch_bounds__(kIrrTexThreads) k_irradiance_texels(const float4* __restrict__ env, int We,
+                                                                 int He, int Wi, int Hi,
+                                                                 float4* __restrict__ part) {
+  __shared__ float4 s_src[kIrrTile][3];
+  long long ntex = (long long)We * He;
+  long long per = (ntex + gridDim.x - 1) / gridDim.x;
+  long long t0 = per * blockIdx.x;
+  long long t1 = t0 + per < ntex ? t0 + per : ntex;
+  int nout = Wi * Hi;
+  // Omega of row y = (2 pi / W)(cos(pi y / H) - cos(pi (y + 1) / H))
+  //               = (4 pi / W) sin(pi (y + 0.5) / H) sin(pi / (2 H))   (product form)
+  float row_k = 4.0f * kPi / We * sinpif(0.5f / He);
+  for (int og = blockIdx.y * kIrrTexThreads * kIrrOutPerThread; og < nout;
+       og += gridDim.y * kIrrTexThreads * kIrrOutPerThread) {
+    // pair p holds outputs og + (2p + h) * kIrrTexThreads + tid, h = 0, 1; an absent output has n = 0
+    float2 nx[2], ny[2], nz[2];
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      float3 a, b;
+      int oa = og + (2 * p) * kIrrTexThreads + threadIdx.x, ob = oa + kIrrTexThreads;
+      a = oa < nout ? texel_dir(oa % Wi, oa / Wi, Wi, Hi) : f3(0, 0, 0);
+      b = ob < nout ? texel_dir(ob % Wi, ob / Wi, Wi, Hi) : f3(0, 0, 0);
+      nx[p] = make_float2(a.x, b.x), ny[p] = make_float2(a.y, b.y), nz[p] = make_float2(a.z, b.z);
+    }
+    Kahan acc[kIrrOutPerThread][4];
+    for (long long base = t0; base < t1; base += kIrrTile) {
+      int cnt = (int)(t1 - base < kIrrTile ? t1 - base : kIrrTile);
+      __syncthreads();
+      for (int q = threadIdx.x; q < cnt; q += kIrrTexThreads) {
+        long long t = base + q;
+        int x = (int)(t % We), y = (int)(t / We);
+        float3 d = texel_dir(x, y, We, He) * (row_k * sinpif((y + 0.5f) / He));
+        float4 L = __ldg(env + t);
+        s_src[q][0] = make_float4(d.x, d.x, d.y, d.y);
+        s_src[q][1] = make_float4(d.z, d.z, L.x, L.x);
+        s_src[q][2] = make_float4(L.y, L.y, L.z, L.z);
+      }
+      __syncthreads();
+      float2 sr[2], sg[2], sb[2], sw[2];
+#pragma unroll
+      for (int p = 0; p < 2; ++p) sr[p] = sg[p] = sb[p] = sw[p] = make_float2(0.0f, 0.0f);
+#pragma unroll 4
+      for (int q = 0; q < cnt; ++q) {
+        const float4 u = s_src[q][0], v = s_src[q][1], z = s_src[q][2];
+        const float2 dx = make_float2(u.x, u.y), dy = make_float2(u.z, u.w), dz = make_float2(v.x, v.y);
+        const float2 Lr = make_float2(v.z, v.w), Lg = make_float2(z.x, z.y), Lb = make_float2(z.z, z.w);
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+          float2 w = __ffma2_rn(nx[p], dx, __ffma2_rn(ny[p], dy, __fmul2_rn(nz[p], dz)));
+          w = make_float2(fmaxf(w.x, 0.0f), fmaxf(w.y, 0.0f));
+          sr[p] = __ffma2_rn(Lr, w, sr[p]);
+          sg[p] = __ffma2_rn(Lg, w, sg[p]);
+          sb[p] = __ffma2_rn(Lb, w, sb[p]);
+          sw[p] = __fadd2_rn(sw[p], w);
+        }
+      }
+#pragma unroll
+      for (int p = 0; p < 2; ++p) {
+        acc[2 * p][0].add(sr[p].x), acc[2 * p][1].add(sg[p].x), acc[2 * p][2].add(sb[p].x);
+        acc[2 * p][3].add(sw[p].x);
+        acc[2 * p + 1][0].add(sr[p].y), acc[2 * p + 1][1].add(sg[p].y), acc[2 * p + 1][2].add(sb[p].y);
+        acc[2 * p + 1][3].add(sw[p].y);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < kIrrOutPerThread; ++r) {
+      int o = og + r * kIrrTexThreads + threadIdx.x;
+      if (o < nout)
+        part[(size_t)blockIdx.x * nout + o] =
+            make_float4(acc[r][0].s - acc[r][0].c, acc[r][1].s - acc[r][1].c,
+                        acc[r][2].s - acc[r][2].c, acc[r][3].s - acc[r][3].c);
+    }
   }
   complete_in_order();
 }
@@ -760,22 +853,33 @@ namespace epbr {
 static epbr_status launch_irradiance(const epbr_env* env, int Wi, int Hi, float4* ws, float4* out, cudaStream_t s,
                                      bool early) {
   const int We = env->width, He = env->height, nout = Wi * Hi;
-  const bool round = We <= kIrrPiece && We % kIrrSeg == 0;
-  // slices of whole row pieces, as even as the three blocks an SM holds allow
-  const long long pieces = (long long)He * ((We + kIrrPiece - 1) / kIrrPiece), room = 3LL * num_sms();
-  const long long each = (pieces + room - 1) / room;
-  const int nb = (int)std::min<long long>(irr_blocks(We, He), (pieces + each - 1) / each);
-  // few slices (a small environment): smaller blocks, several per slice
-  const int threads = nb >= num_sms() ? kIrrThreads : 128, passes = (nout + threads - 1) / threads;
-  const int gy = (int)std::min<long long>(std::min(passes, 65535), std::max<long long>(1, room / nb));
-  const size_t smem = irr_shared(nullptr, std::min(We, kIrrPiece)).bytes;
   epbr_status st;
-  void (*k)(const float4*, int, int, int, int, float4*) = round ? k_irradiance_part<true> : k_irradiance_part<false>;
-  if ((st = allow_shared(k, irr_shared(nullptr, kIrrPiece).bytes, "irradiance"))) return st;
-  if ((st = launched(launch_kernel(k, dim3(nb, gy), dim3(threads), smem, s, early, (const float4*)env->texels, We, He, Wi, Hi,
-                                   ws),
-                     "k_irradiance_part")))
-    return st;
+  int nb;
+  const bool round = We <= kIrrPiece && We % kIrrSeg == 0;
+  if (!round && We < kIrrNarrow) {
+    nb = irr_blocks(We, He);
+    const int groups = (nout + kIrrTexThreads * kIrrOutPerThread - 1) / (kIrrTexThreads * kIrrOutPerThread);
+    const int gy = (int)std::min<long long>(groups, std::max<long long>(1, 8LL * num_sms() / nb));
+    if ((st = launched(launch_kernel(k_irradiance_texels, dim3(nb, gy), dim3(kIrrTexThreads), 0, s, early,
+                                     (const float4*)env->texels, We, He, Wi, Hi, ws),
+                       "k_irradiance_texels")))
+      return st;
+  } else {
+    // slices of whole row pieces, as even as the three blocks an SM holds allow
+    const long long pieces = (long long)He * ((We + kIrrPiece - 1) / kIrrPiece), room = 3LL * num_sms();
+    const long long each = (pieces + room - 1) / room;
+    nb = (int)std::min<long long>(irr_blocks(We, He), (pieces + each - 1) / each);
+    // few slices (a small environment): smaller blocks, several per slice
+    const int threads = nb >= num_sms() ? kIrrThreads : 128, passes = (nout + threads - 1) / threads;
+    const int gy = (int)std::min<long long>(std::min(passes, 65535), std::max<long long>(1, room / nb));
+    const size_t smem = irr_shared(nullptr, std::min(We, kIrrPiece)).bytes;
+    void (*k)(const float4*, int, int, int, int, float4*) = round ? k_irradiance_part<true> : k_irradiance_part<false>;
+    if ((st = allow_shared(k, irr_shared(nullptr, kIrrPiece).bytes, "irradiance"))) return st;
+    if ((st = launched(launch_kernel(k, dim3(nb, gy), dim3(threads), smem, s, early, (const float4*)env->texels, We, He,
+                                     Wi, Hi, ws),
+                       "k_irradiance_part")))
+      return st;
+  }
   k_irradiance_final<<<(unsigned)(((long long)nout * 32 + 255) / 256), 256, 0, s>>>(ws, nb, nout, out);
   return check_launch("k_irradiance_final");
 }
