@@ -156,9 +156,19 @@ SHADOW = {"size": 512, "fov_deg": 90.0, "bias_const": 0.02, "bias_slope": 0.01}
 MESH = {"n_lat": 16, "n_lon": 32, "ground_cells": 64, "near": 0.05}
 RASTER_LAUNCHES = 3  # triangles, queued boxes, resolve (the key reset is a memset)
 SHADOW_MAP_LAUNCHES = 2  # per group of lights, after one fill: triangles, queued boxes
-SHADOW_MAP_GROUP = 9     # lights that the workspace of this mesh and map size has room for
 SURFELS = {"per_sphere": 4000, "ground": 400000, "overlap": 1.2, "seed": 11, "near": 0.05, "tolerance": 0.01}
 SURFEL_LAUNCHES = 5  # count, list ranges, fill, tiles, heavy tiles (the count reset is a memset)
+
+
+def shadow_map_launches(ep, triangles: int, size: int, maps: int) -> int:
+    """Kernels of one epbr_shadow_maps call: the fill, then two per group of lights.  A group has as many
+    lights as the workspace holds set-ups (64 B per triangle) and queue entries (8 B) for, less 768 B of
+    counters and alignment; 8 at least, 32 at most."""
+    if maps == 0 or triangles == 0:
+        return min(maps, 1)
+    room = ep.epbr_shadow_maps_workspace_size(triangles, size) - 768
+    group = min(32, max(room // (72 * triangles), 8), (2**31 - 1) // triangles)
+    return 1 + SHADOW_MAP_LAUNCHES * -(-maps // group)
 
 
 def compose_flops(sc, g, n_lights) -> tuple[float, dict]:
@@ -585,7 +595,7 @@ def run_gpu(args):
         compose(gb, shp, hdr, ldr, lights, record)
 
     launches_per_step = 3 + (BLOOM_LAUNCHES if args.bloom else 0) + (RASTER_LAUNCHES if args.mesh else 0) + \
-        (SURFEL_LAUNCHES if args.surfels else 0) + (1 + SHADOW_MAP_LAUNCHES * -(-len(scams) // SHADOW_MAP_GROUP) if smaps_dev else 0)
+        (SURFEL_LAUNCHES if args.surfels else 0) + (shadow_map_launches(ep, smesh.struct.num_triangles, SHADOW["size"], len(scams)) if smaps_dev else 0)
     with torch.cuda.stream(stream):
         for _ in range(max(3, args.warmup)):
             step()
@@ -784,7 +794,7 @@ def run_gpu(args):
     if smaps_dev:
         line["shadow_maps"] = {"ms": statistics.mean(a.elapsed_time(b) for a, b in ev_smaps), "maps": len(scams),
                                "size": SHADOW["size"], "triangles": smesh.struct.num_triangles,
-                               "launches": 1 + SHADOW_MAP_LAUNCHES * -(-len(scams) // SHADOW_MAP_GROUP)}
+                               "launches": shadow_map_launches(ep, smesh.struct.num_triangles, SHADOW["size"], len(scams))}
     if args.surfels:
         line["surfels"] = {"ms": statistics.mean(a.elapsed_time(b) for a, b in ev_raster), "surfels": len(srec),
                            "launches": SURFEL_LAUNCHES, **SURFELS}
