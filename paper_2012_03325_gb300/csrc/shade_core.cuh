@@ -254,11 +254,7 @@ __device__ __forceinline__ LightTerms light_terms(const Px& s, const Direct& d, 
   float hh = fmaf(h.x, h.x, fmaf(h.y, h.y, h.z * h.z));  // |s|^2
   float den = fmaf(nsa, nsa, c2);
   float xx = fmaf(-0.5f, sqrt_ftz(hh), 1.0f);  // 1 - v.h, v.h = |l + v| / 2
-#ifdef EPBR_FC_POW5
-  float x2 = xx * xx, fc = x2 * x2 * xx;
-#else
   float fc = ex2_ftz(5.0f * lg2_ftz(fabsf(xx)));  // (1 - v.h)^5 (|xx|: v.h may round above 1)
-#endif
   float w = rs * rs * nlc;  // (n.l) / d^2
   float spec = hh * hh * rcp_ftz(den * den * fmaf(nlc, d.omk, d.k));
   LightTerms t;
