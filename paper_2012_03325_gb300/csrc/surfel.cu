@@ -208,10 +208,14 @@ __device__ __forceinline__ SurfelCellRange surfel_cells(const SurfelGrid& g, uin
 // more than 1.5 times a warp's share of all tiles' entries (at most 2/3 of the warps can then own one),
 // and kHeavyMin entries.  Its list is cut into units of a 16th of the share, kHeavyUnit at least, so there are
 // at most about 16 units per warp.  Times (us) with the line at 1, 1.5, 2 and 3 shares: 1080p surfels of 1.2 M
-// in three scenes 267 / 252, 256 / 247, 259 / 252, 282 / 252; 2560 x 1440 346, 344, 331, 332; 300,000 surfels of
-// 30 pixels in the middle tenth of 1080p 9540, 10100, 11200, 12700.  kHeavyMin 64, 96, 128: 10,000 surfels
-// of 3 pixels over 64 x 64 pixels 56, 51, 63; 2809 surfels over 128 x 96 52, 53, 49 (45 never shared out).
-constexpr unsigned kHeavyMin = 96, kHeavyUnit = 32;
+// in two scenes 267, 256, 259, 282 and 252, 247, 252, 252; 300,000 surfels of 30 pixels in the middle tenth of
+// 1080p 9540, 10100, 11200, 12700.  kHeavyMin 64, 96, 128: 70,000 surfels over 128 x 96 57, 58, 58; 160,000
+// over 300 x 200 72, 65, 81.  The second pass costs about 13 us, so the heavy tiles are shared out only when
+// the longest list has more than 3 shares and kHeavyTrigger entries: else each is left to its warp
+// (1992 x 195, 25,000 surfels, longest list 150: 51 us instead of 68; 1080p, longest 2.2 shares: 236 instead
+// of 247; but 1080p, longest 3.4 shares: 294 instead of 257, longest 1478 entries, 21 shares: 202 instead of
+// 102).
+constexpr unsigned kHeavyMin = 96, kHeavyUnit = 32, kHeavyTrigger = 288;
 constexpr unsigned kHeavyFlag = 1u << 31;  // of a level-0 cell's count (at most 2^28): its tile is heavy
 
 struct SurfelHeader {  // all zero before k_surfel_count
@@ -219,15 +223,14 @@ struct SurfelHeader {  // all zero before k_surfel_count
   unsigned long long work;   // entries of all tiles' lists together
   unsigned listed;           // entries of the list
   unsigned used;             // of them, those given to cells
-  unsigned pad[2];
+  unsigned longest;          // entries of the longest list of a heavy tile
+  unsigned pad;
 };
 
 // A heavy tile, from the end of the workspace backwards, as far as the list leaves room (a tile without
-// room is not heavy).
+// room is not heavy).  Its nearest depths (as bits) and sums are gathered in the G-buffer's own pixels.
 struct SurfelHeavy {
-  unsigned depth[32];  // per pixel: bits of the nearest depth
-  float4 a[32], n[32];
-  float w[32];         // the sums
+  float w[32];            // per pixel: the number of blended surfels
   unsigned first, units;  // its first unit of all heavy tiles' (ascending), their number
   unsigned tile, entries;
   unsigned done, pad[3];  // units whose surfels are in the sums
@@ -235,10 +238,15 @@ struct SurfelHeavy {
 
 struct HeavyRule {
   unsigned limit, unit;  // a tile with more than `limit` entries is heavy; entries per unit
+  unsigned trigger;      // the heavy tiles are shared out when one has more entries than this
 };
 __device__ __forceinline__ HeavyRule heavy_rule(const SurfelHeader* h, unsigned warps) {
   const unsigned share = (unsigned)fminf(__fdividef((float)__ldcg(&h->work), (float)warps), 268435456.0f);
-  return HeavyRule{max(kHeavyMin, share + share / 2), max(kHeavyUnit, (share / 16 + 31) & ~31u)};
+  return HeavyRule{max(kHeavyMin, share + share / 2), max(kHeavyUnit, (share / 16 + 31) & ~31u), max(kHeavyTrigger, 3 * share)};
+}
+__device__ __forceinline__ bool heavy_shared(const SurfelHeader* h, unsigned warps) {
+  const unsigned longest = __ldcg(&h->longest);
+  return longest > 0 && longest > heavy_rule(h, warps).trigger;
 }
 __device__ __forceinline__ SurfelHeavy* heavy_at(char* end, unsigned slot) { return (SurfelHeavy*)end - (slot + 1); }
 __device__ __forceinline__ unsigned heavy_room(const SurfelHeader* h, const unsigned* list, const char* end) {
@@ -297,27 +305,70 @@ __global__ void __launch_bounds__(256) k_surfel_count(const float4* __restrict__
   }
 }
 
-// cursor[k] = the first list entry of cell k.
+__device__ __forceinline__ float4* surfel_a(const GbufDev& out, int x, int y) {
+  return (float4*)(const_cast<char*>(out.rt[0]) + (size_t)y * out.pitch[0]) + x;
+}
+__device__ __forceinline__ float4* surfel_n(const GbufDev& out, int x, int y) {
+  return (float4*)(const_cast<char*>(out.rt[1]) + (size_t)y * out.pitch[1]) + x;
+}
+__device__ __forceinline__ float* surfel_depth(const GbufDev& out, int x, int y) {
+  return (float*)(const_cast<char*>(out.rt[3]) + (size_t)y * out.pitch[3]) + x;
+}
+
+// Whether tile k is heavy, and its entry if so.
+__device__ __forceinline__ void surfel_weigh(int k, unsigned* __restrict__ counts, SurfelHeader* __restrict__ head,
+                                             const SurfelGrid& g, const unsigned* list, char* end, unsigned warps,
+                                             const GbufDev& out) {
+  const int y = k / g.nx[0], x = k - y * g.nx[0];
+  unsigned entries = __ldcg(counts + g.at(k));  // on all levels; only this thread sets the flag of this cell
+  const unsigned own = entries;
+#pragma unroll
+  for (int l = 1; l < kSurfelLevels; ++l)
+    if (l < g.levels) entries += __ldcg(counts + g.at(g.first[l] + (y >> l) * g.nx[l] + (x >> l)));
+  const HeavyRule rule = heavy_rule(head, warps);
+  if (entries <= rule.limit) return;
+  const unsigned units = (entries + rule.unit - 1) / rule.unit;
+  const unsigned long long old = atomicAdd(&head->heavy, ((unsigned long long)units << 32) | 1ull);
+  const unsigned slot = (unsigned)old;
+  if (slot >= heavy_room(head, list, end)) return;
+  atomicMax(&head->longest, entries);
+  SurfelHeavy* h = heavy_at(end, slot);
+  for (int q = 0; q < 32; ++q) {
+    const int px = x * kTileW + (q & 7), py = y * kTileH + (q >> 3);
+    h->w[q] = 0.0f;
+    if (px >= out.W || py >= out.H) continue;
+    *surfel_a(out, px, py) = *surfel_n(out, px, py) = make_float4(0, 0, 0, 0);
+    *(unsigned*)surfel_depth(out, px, py) = 0xffffffffu;
+  }
+  h->first = (unsigned)(old >> 32);
+  h->units = units;
+  h->tile = k;
+  h->entries = entries;
+  h->done = 0;
+  counts[g.at(k)] = own | kHeavyFlag;
+}
+
+// cursor[k] = the first list entry of cell k.  The blocks after those of the cells weigh the tiles.
 template <bool HEAVY>
 __global__ void __launch_bounds__(256) k_surfel_alloc(unsigned* __restrict__ counts, int cells,
                                                       unsigned* __restrict__ cursor, SurfelHeader* __restrict__ head,
                                                       const __grid_constant__ SurfelGrid g, const unsigned* list, char* end,
-                                                      unsigned warps) {
+                                                      unsigned warps, GbufDev out) {
   __shared__ unsigned s_warp[8];
   __shared__ unsigned s_base;
   griddep_wait();
   griddep_launch_dependents();
-  const int k = blockIdx.x * 256 + threadIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const unsigned n = k < cells ? __ldcg(counts + g.at(k)) : 0u;
-  unsigned entries = n;  // of a tile (a cell of level 0), on all levels
-  HeavyRule rule;
-  if (HEAVY && k < g.first[1]) {
-    rule = heavy_rule(head, warps);
-    const int y = k / g.nx[0], x = k - y * g.nx[0];
-#pragma unroll
-    for (int l = 1; l < kSurfelLevels; ++l)
-      if (l < g.levels) entries += __ldcg(counts + g.at(g.first[l] + (y >> l) * g.nx[l] + (x >> l)));
+  int k = blockIdx.x * 256 + threadIdx.x;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (HEAVY) {
+    const int blocks = (cells + 255) / 256;
+    if (blockIdx.x >= blocks) {
+      k -= blocks * 256;
+      if (k < g.first[1]) surfel_weigh(k, counts, head, g, list, end, warps, out);
+      return;
+    }
   }
+  const unsigned n = k < cells ? __ldcg(counts + g.at(k)) & ~kHeavyFlag : 0u;
   unsigned incl = n;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -338,27 +389,6 @@ __global__ void __launch_bounds__(256) k_surfel_alloc(unsigned* __restrict__ cou
   }
   __syncthreads();
   if (k < cells) cursor[g.at(k)] = s_base + s_warp[warp] + incl - n;
-  if (HEAVY && k < g.first[1]) {
-    if (entries > rule.limit) {
-      const unsigned units = (entries + rule.unit - 1) / rule.unit;
-      const unsigned long long old = atomicAdd(&head->heavy, ((unsigned long long)units << 32) | 1ull);
-      const unsigned slot = (unsigned)old;
-      if (slot < heavy_room(head, list, end)) {
-        SurfelHeavy* h = heavy_at(end, slot);
-        for (int q = 0; q < 32; ++q) {
-          h->depth[q] = 0xffffffffu;
-          h->a[q] = h->n[q] = make_float4(0, 0, 0, 0);
-          h->w[q] = 0.0f;
-        }
-        h->first = (unsigned)(old >> 32);
-        h->units = units;
-        h->tile = k;
-        h->entries = entries;
-        h->done = 0;
-        counts[g.at(k)] = n | kHeavyFlag;  // read by no other thread of this kernel
-      }
-    }
-  }
 }
 
 // Afterwards cursor[k] is the end of cell k's range.
@@ -621,9 +651,8 @@ __device__ __forceinline__ void surfel_walk(SurfelWarp& st, const float4* __rest
 // The means of a pixel (w surfels, the sums a and n) as the FP32 G-buffer.
 __device__ __forceinline__ void surfel_store(const GbufDev& out, float* __restrict__ weight, long long weight_pitch, int x,
                                              int y, float w, float4 a, float4 n, float depth) {
-  float4* rt0 = (float4*)(const_cast<char*>(out.rt[0]) + (size_t)y * out.pitch[0]) + x;
-  float4* rt1 = (float4*)(const_cast<char*>(out.rt[1]) + (size_t)y * out.pitch[1]) + x;
-  float* dep = (float*)(const_cast<char*>(out.rt[3]) + (size_t)y * out.pitch[3]) + x;
+  float4 *rt0 = surfel_a(out, x, y), *rt1 = surfel_n(out, x, y);
+  float* dep = surfel_depth(out, x, y);
   if (weight) ((float*)((char*)weight + (size_t)y * weight_pitch))[x] = w;
   if (w == 0.0f) {
     *rt0 = make_float4(0, 0, 0, 0);
@@ -653,8 +682,8 @@ template <int PASS>
 __device__ __forceinline__ void surfel_runs(SurfelWarp& st, const SurfelArgs& s, const SurfelCam& cam, const SurfelGrid& g,
                                             unsigned warp, unsigned warps, int lane, const GbufDev& out,
                                             float* __restrict__ weight, long long weight_pitch) {
+  if (!heavy_shared(s.head, s.warps)) return;
   const unsigned long long heavy = __ldcg(&s.head->heavy);
-  if (heavy == 0) return;
   const unsigned total = (unsigned)(heavy >> 32), slots = min((unsigned)heavy, heavy_room(s.head, s.list, s.end));
   const unsigned unit = heavy_rule(s.head, s.warps).unit, run = (total + 2 * warps - 1) / (2 * warps);
   for (unsigned u0 = warp * run; u0 < total; u0 += warps * run) {
@@ -682,8 +711,9 @@ __device__ __forceinline__ void surfel_runs(SurfelWarp& st, const SurfelArgs& s,
       SurfelPixel p;
       p.clear();
       p.dmin = __int_as_float(0x7f800000);
+      const bool inside = x < cam.W && y < cam.H;
       if (PASS == kBlend) {
-        const unsigned bits = __ldcg(h->depth + lane);
+        const unsigned bits = inside ? __ldcg((const unsigned*)surfel_depth(out, x, y)) : 0xffffffffu;
         if (bits != 0xffffffffu) p.dmin = __uint_as_float(bits);
         p.lim = __fmul_rn(p.dmin, cam.f);
       }
@@ -691,11 +721,11 @@ __device__ __forceinline__ void surfel_runs(SurfelWarp& st, const SurfelArgs& s,
       surfel_walk<PASS>(st, s.rec, s.boxes, cam, g, t, s.list, k0 * unit, min(k1 * unit, __ldcg(&h->entries)), lane, p);
       __syncwarp();
       if (PASS == kNearest) {
-        if (st.nearest[lane] != 0xffffffffu) atomicMin(h->depth + lane, st.nearest[lane]);
+        if (st.nearest[lane] != 0xffffffffu) atomicMin((unsigned*)surfel_depth(out, x, y), st.nearest[lane]);
       } else {
         if (p.w > 0.0f) {
-          atomicAdd(h->a + lane, make_float4(p.a0, p.a1, p.a2, p.a3));
-          atomicAdd(h->n + lane, make_float4(p.n0, p.n1, p.n2, p.n3));
+          atomicAdd(surfel_a(out, x, y), make_float4(p.a0, p.a1, p.a2, p.a3));
+          atomicAdd(surfel_n(out, x, y), make_float4(p.n0, p.n1, p.n2, p.n3));
           atomicAdd(h->w + lane, p.w);
         }
         __threadfence();
@@ -705,9 +735,9 @@ __device__ __forceinline__ void surfel_runs(SurfelWarp& st, const SurfelArgs& s,
         done = __shfl_sync(0xffffffffu, done, 0);
         if (done + (k1 - k0) == units) {  // the tile's last units
           __threadfence();
-          if (x < cam.W && y < cam.H)
-            surfel_store(out, weight, weight_pitch, x, y, __ldcg(h->w + lane), __ldcg(h->a + lane), __ldcg(h->n + lane),
-                         p.dmin);
+          if (inside)
+            surfel_store(out, weight, weight_pitch, x, y, __ldcg(h->w + lane), __ldcg(surfel_a(out, x, y)),
+                         __ldcg(surfel_n(out, x, y)), p.dmin);
         }
       }
       __syncwarp();
@@ -726,6 +756,8 @@ __global__ void __launch_bounds__(32 * kSurfelTileWarps)
     k_surfel_tile(const __grid_constant__ SurfelArgs s, const SurfelCam cam, const __grid_constant__ SurfelGrid g,
                   int heavy_rows, GbufDev out, float* __restrict__ weight, long long weight_pitch) {
   __shared__ __align__(16) SurfelWarp s_all[kSurfelTileWarps];
+  // k_surfel_alloc, which writes the header, was complete before k_surfel_fill let this kernel begin
+  if (HEAVY && blockIdx.y < heavy_rows && !heavy_shared(s.head, s.warps)) return;
   griddep_wait();
   if (HEAVY) griddep_launch_dependents();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -738,8 +770,11 @@ __global__ void __launch_bounds__(32 * kSurfelTileWarps)
   const int tx = (blockIdx.x * kSurfelTileWarps + warp) * kTileW, ty = (blockIdx.y - heavy_rows) * kTileH;
   if (tx >= cam.W) return;  // warp-uniform, no block barrier below
   const int x = tx + (lane & 7), y = ty + (lane >> 3);
-  const SurfelTile t = surfel_tile(g, tx, ty, lane, s.counts, s.cursor);
-  if (HEAVY && (__shfl_sync(0xffffffffu, t.n, 0) & kHeavyFlag)) return;
+  SurfelTile t = surfel_tile(g, tx, ty, lane, s.counts, s.cursor);
+  if (HEAVY && (__shfl_sync(0xffffffffu, t.n, 0) & kHeavyFlag)) {
+    if (heavy_shared(s.head, s.warps)) return;
+    t.n &= ~kHeavyFlag;
+  }
   st.nearest[lane] = 0xffffffffu;
   st.ray[lane] = surfel_ray(cam, x, y);
   SurfelPixel p;
@@ -762,6 +797,8 @@ __global__ void __launch_bounds__(32 * kSurfelTileWarps, 6)
     k_surfel_heavy(const __grid_constant__ SurfelArgs s, const SurfelCam cam, const __grid_constant__ SurfelGrid g,
                    GbufDev out, float* __restrict__ weight, long long weight_pitch) {
   __shared__ __align__(16) SurfelWarp s_all[kSurfelTileWarps];
+  // the header, as in k_surfel_tile; one block waits, so that this kernel is not complete before the tiles
+  if (!heavy_shared(s.head, s.warps) && blockIdx.x > 0) return;
   griddep_wait();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   surfel_runs<kBlend>(s_all[warp], s, cam, g, blockIdx.x * kSurfelTileWarps + warp, gridDim.x * kSurfelTileWarps, lane, out,
@@ -776,7 +813,7 @@ struct SurfelLayout {
 };
 
 // The workspace: the header, cell counts and cursors, 8 bytes of box and kSurfelCells
-// list entries per surfel; heavy tiles (1312 bytes each) from its end down to the entries that are used.  `bytes` is the size callers have always been told, 40 B per pixel, 4 B
+// list entries per surfel; heavy tiles (160 bytes each) from its end down to the entries that are used.  `bytes` is the size callers have always been told, 40 B per pixel, 4 B
 // per column and row, 104 B per surfel and 8 B per 1024 of them: the list takes 96 B per surfel, the
 // cells less than 4 B per pixel plus 1 KB.
 static SurfelLayout surfel_layout(long long N, int W, int H) {
@@ -799,8 +836,10 @@ static SurfelLayout surfel_layout(long long N, int W, int H) {
   l.head = 0;
   l.counts = sizeof(SurfelHeader);  // reset together
   g.stride = 1;
+  const size_t room = sizeof(SurfelHeavy) * (size_t)g.first[1] + 1024;
   // few cells: their counters apart, up to kSurfelSpread words, as far as the 40 B per pixel hold both arrays
-  while (g.stride < 32 && 2 * cells * g.stride <= kSurfelSpread && 2 * 8 * cells * g.stride + 1024 <= 40 * px) g.stride *= 2;
+  // and the heavy tiles
+  while (g.stride < 32 && 2 * cells * g.stride <= kSurfelSpread && 2 * 8 * cells * g.stride + room <= 40 * px) g.stride *= 2;
   l.counters = cells * g.stride;
   l.cursor = align256(l.counts + 4 * l.counters);
   l.boxes = l.cursor + align256(4 * l.counters);
@@ -875,13 +914,13 @@ extern "C" epbr_status epbr_surfel_gbuffer(const epbr_surfels* surfels, const ep
   const SurfelArgs a = {rec, boxes, counts, cursor, list, head, ws + l.bytes, (unsigned)(heavy_blocks * kSurfelTileWarps)};
   cudaError_t e = cudaSuccess;
   if (N > 0) {
-    const dim3 per_surfel((N + 255) / 256), per_cell((cells + 255) / 256);
+    const dim3 per_surfel((N + 255) / 256), per_cell((cells + 255) / 256 + (heavy ? (g.first[1] + 255) / 256 : 0));
     if (heavy)
       k_surfel_count<true><<<per_surfel, 256, 0, s>>>(rec, N, sc, g, boxes, counts, head);
     else
       k_surfel_count<false><<<per_surfel, 256, 0, s>>>(rec, N, sc, g, boxes, counts, head);
     e = launch_kernel(heavy ? k_surfel_alloc<true> : k_surfel_alloc<false>, per_cell, dim3(256), 0, s, true, counts, cells,
-                      cursor, head, g, (const unsigned*)list, a.end, a.warps);
+                      cursor, head, g, (const unsigned*)list, a.end, a.warps, gd);
     if (e == cudaSuccess)
       e = launch_kernel(k_surfel_fill, per_surfel, dim3(256), 0, s, true, (const uint2*)boxes, N, g, cursor, list);
   }

@@ -41,7 +41,7 @@ def cloud(seed, W, H, n, px, spread, slant=0.3):
 @pytest.mark.parametrize("W,H,n,px,spread,tol", [
     (8, 4, 256, 1.0, 0.6, 0.01), (8, 4, 257, 1.0, 0.6, 0.01), (8, 4, 5000, 0.6, 0.8, 0.0), (7, 3, 2000, 8.0, 0.5, 0.02),
     (24, 12, 900, 2.0, 0.1, 0.01), (64, 64, 300, 60.0, 0.1, 0.01), (64, 64, 20000, 2.5, 1.0, 0.01),
-    (64, 64, 6000, 30.0, 1.0, 0.05), (200, 120, 4000, 0.7, 0.0, 0.01), (200, 120, 3000, 9.0, 0.02, 0.0),
+    (64, 64, 6000, 30.0, 1.0, 0.05), (64, 64, 6000, 200.0, 0.0, 0.01), (200, 120, 4000, 0.7, 0.0, 0.01), (200, 120, 3000, 9.0, 0.02, 0.0),
     (333, 77, 10000, 3.0, 0.05, 0.01), (1, 40, 1000, 1.5, 1.0, 0.01), (300, 1, 3000, 0.5, 1.0, 0.01)])
 def test_few_tiles(W, H, n, px, spread, tol):
     check(W, H, cloud(W + n, W, H, n, px, spread), tol)
