@@ -445,6 +445,12 @@ constexpr int kPrefilterMaxSamples = 2048;
 constexpr int kPrefilterThreads = 256;
 constexpr int kPrefilterTexels = 2;  // texels per thread: a block shades a segment of up to 512 texels of a row
 constexpr int kPrefilterSeg = kPrefilterThreads * kPrefilterTexels;
+// Twice the threads and segment, one block per SM, where level 1 has rows of 1024 to 2048 texels (columns shifted
+// by whole texels) and the records of a row, now made once or twice, are many: 2048 x 1024, 256 / 512 threads (us): 8
+// levels 256, 512, 1024, 2048 samples 544 / 558, 1054 / 1037, 2067 / 2004, 4562 / 3933; 3 levels 1024 samples
+// 1623 / 1526; 2048 x 300 920 / 818; but 1024 x 512, 8 levels, 1024 samples 529 / 569 and 8192 x 256, 512
+// samples 1181 / 1321.
+constexpr int kPrefilterWideMin = 1024, kPrefilterWideMax = 2048, kPrefilterWideSamples = 512;
 // Segments are halved down to kPrefilterMinSeg texels until a launch has kPrefilterFill blocks per SM (each
 // block makes its row's records anew).  Prefilter (us) with the shortest segment 64, 128, 256 or 512 texels: 2048 x
 // 64, 8 levels, 1024 samples 224, 252, 357, 315; 512 x 256, 6 levels, 512 samples 121, 103, 98, 98; 2048 x 1024
@@ -474,14 +480,14 @@ __device__ __forceinline__ float2 prefilter_src_xy(float3 l, int W0, int H0) {
 // positions; the sort keys (N unsigned) occupy the weights' space until the records are written.
 struct PrefilterShared {
   int base[kPrefilterMaxSamples / 32 + 1];
-  float wsum[kPrefilterThreads / 32];
+  float wsum[16];
 };
 
 // The samples of row j of level m as records in order of source row (a deterministic bitonic sort of
 // (source row, sample) keys), by a whole block: `emit(position, sample (.z = n.l), source x, y for texel 0)`
 // writes a record.  Returns the number of kept samples and their weight sum sum_k n.l_k (the same for every
 // texel of the level).
-template <typename Emit>
+template <int THREADS, typename Emit>
 __device__ __forceinline__ int prefilter_records(PrefilterShared& sh, unsigned* s_key, unsigned short* s_pos, int m,
                                                  int M, int j, int W, int H, int W0, int H0, int N, float& wsum,
                                                  Emit emit) {
@@ -491,7 +497,7 @@ __device__ __forceinline__ int prefilter_records(PrefilterShared& sh, unsigned* 
   const int groups = (N + 31) / 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // kept samples per group of 32, then an exclusive prefix over the groups (sample order)
-  for (int gi = warp; gi < groups; gi += kPrefilterThreads / 32) {
+  for (int gi = warp; gi < groups; gi += THREADS / 32) {
     int sidx = gi * 32 + lane;
     bool keep = sidx < N && prefilter_sample(sidx, a2, invN).z > 0.0f;
     unsigned bal = __ballot_sync(0xffffffffu, keep);
@@ -516,7 +522,7 @@ __device__ __forceinline__ int prefilter_records(PrefilterShared& sh, unsigned* 
   const float3 T = f3(-cp0, 0.0f, -sp0);
   const float3 B = cross3(n, T);
   // pass A: each kept sample's source row, as a sort key
-  for (int gi = warp; gi < groups; gi += kPrefilterThreads / 32) {
+  for (int gi = warp; gi < groups; gi += THREADS / 32) {
     int sidx = gi * 32 + lane;
     float4 e = sidx < N ? prefilter_sample(sidx, a2, invN) : make_float4(0, 0, 0, 0);
     bool keep = sidx < N && e.z > 0.0f;
@@ -530,11 +536,11 @@ __device__ __forceinline__ int prefilter_records(PrefilterShared& sh, unsigned* 
   }
   int P = 1;
   while (P < ns) P <<= 1;
-  for (int q = ns + tid; q < P; q += kPrefilterThreads) s_key[q] = 0xffffffffu;
+  for (int q = ns + tid; q < P; q += THREADS) s_key[q] = 0xffffffffu;
   __syncthreads();
   for (int k = 2; k <= P; k <<= 1) {
     for (int jj = k >> 1; jj > 0; jj >>= 1) {
-      for (int q = tid; q < P; q += kPrefilterThreads) {
+      for (int q = tid; q < P; q += THREADS) {
         const int o = q ^ jj;
         if (o > q) {
           const unsigned a = s_key[q], b = s_key[o];
@@ -547,11 +553,11 @@ __device__ __forceinline__ int prefilter_records(PrefilterShared& sh, unsigned* 
       __syncthreads();
     }
   }
-  for (int q = tid; q < ns; q += kPrefilterThreads) s_pos[s_key[q] & 0xffffu] = (unsigned short)q;
+  for (int q = tid; q < ns; q += THREADS) s_pos[s_key[q] & 0xffffu] = (unsigned short)q;
   __syncthreads();  // the keys are dead from here: their space takes the records
   // pass B: the records at their sorted positions; the weights summed in sample order
   float wpart = 0.0f;
-  for (int gi = warp; gi < groups; gi += kPrefilterThreads / 32) {
+  for (int gi = warp; gi < groups; gi += THREADS / 32) {
     int sidx = gi * 32 + lane;
     float4 e = sidx < N ? prefilter_sample(sidx, a2, invN) : make_float4(0, 0, 0, 0);
     bool keep = sidx < N && e.z > 0.0f;
@@ -567,7 +573,7 @@ __device__ __forceinline__ int prefilter_records(PrefilterShared& sh, unsigned* 
   __syncthreads();
   wsum = 0.0f;
 #pragma unroll
-  for (int w = 0; w < kPrefilterThreads / 32; ++w) wsum += sh.wsum[w];
+  for (int w = 0; w < THREADS / 32; ++w) wsum += sh.wsum[w];
   return ns;
 }
 
@@ -577,11 +583,11 @@ __device__ __forceinline__ int prefilter_records(PrefilterShared& sh, unsigned* 
 // row.  Samples are visited in order of their source row so that consecutive samples read the
 // same two rows, which stay in L1.  A plain FP32 sum takes 64 samples, compensated sums take the
 // plain ones and the shares.
-template <bool INT_SHIFT>
+template <bool INT_SHIFT, int THREADS>
 __device__ __forceinline__ void prefilter_segment(const MapDev& src, const ChainDev& ch, int N, int seg) {
   extern __shared__ __align__(16) float4 s_pf[];
   __shared__ PrefilterShared sh;
-  __shared__ float3 s_sum[kPrefilterThreads * 2];  // the shares' sums
+  __shared__ float3 s_sum[THREADS * 2];  // the shares' sums
   float4* s_w = s_pf;
   int2* s_xy = (int2*)(s_pf + N);
   unsigned short* s_pos = (unsigned short*)(s_xy + N);
@@ -593,7 +599,7 @@ __device__ __forceinline__ void prefilter_segment(const MapDev& src, const Chain
   const int W0 = src.W, H0 = src.H;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   float wsum;
-  const int ns = prefilter_records(
+  const int ns = prefilter_records<THREADS>(
       sh, (unsigned*)s_pf, s_pos, m, ch.M, j, W, H, W0, H0, N, wsum,
       [&](int p, float4 e, float2 xy) {
         const float xf = floorf(xy.x), yf = floorf(xy.y);
@@ -615,7 +621,8 @@ __device__ __forceinline__ void prefilter_segment(const MapDev& src, const Chain
     // their sums at the end.
     // A segment of at most 256 texels leaves warps over: these take shares of the samples (`split`).
     const int cols = (min(W - i0, seg) + 63) / 64;  // warps side by side
-    const int across = cols > 4 ? 8 : (cols > 2 ? 4 : cols), split = warp / across, splits = 8 / across;
+    const int across = cols > 8 ? 16 : (cols > 4 ? 8 : (cols > 2 ? 4 : cols));
+    const int split = warp / across, splits = THREADS / 32 / across;
     const int t = lane >> 1, dl = lane & 1;
     const int wbase = i0 + (warp - split * across) * 64;
     int col[4];
@@ -691,16 +698,16 @@ __device__ __forceinline__ void prefilter_segment(const MapDev& src, const Chain
   }
   // a thread per texel, or per texel and share of the samples where the segment has at most 128
   const int n = min(W - i0, seg);
-  const int across = n > 128 ? 256 : (n > 64 ? 128 : (n > 32 ? 64 : 32)), split = tid / across;
-  const int splits = kPrefilterThreads / across, me = tid - split * across;
+  const int across = n > 128 ? THREADS : (n > 64 ? 128 : (n > 32 ? 64 : 32)), split = tid / across;
+  const int splits = THREADS / across, me = tid - split * across;
   int ii[kPrefilterTexels];
   bool on[kPrefilterTexels];  // block-uniform: whether the segment has a texel group c
   Kahan3 acc[kPrefilterTexels];
   float3 part[kPrefilterTexels];
 #pragma unroll
   for (int c = 0; c < kPrefilterTexels; ++c) {
-    on[c] = c * kPrefilterThreads < n;
-    ii[c] = min(i0 + c * kPrefilterThreads + me, W - 1);  // duplicates of the last texel are not stored
+    on[c] = c * THREADS < n;
+    ii[c] = min(i0 + c * THREADS + me, W - 1);  // duplicates of the last texel are not stored
     part[c] = f3(0, 0, 0);
   }
   auto sum = [&](auto whole) {
@@ -748,7 +755,7 @@ __device__ __forceinline__ void prefilter_segment(const MapDev& src, const Chain
   }
 #pragma unroll
   for (int c = 0; c < kPrefilterTexels; ++c) {
-    const int i = i0 + c * kPrefilterThreads + me;
+    const int i = i0 + c * THREADS + me;
     if (on[c] && i < W) {
       Kahan3 v = acc[c];
       v.add(part[c]);
@@ -764,11 +771,11 @@ __device__ __forceinline__ void prefilter_segment(const MapDev& src, const Chain
 // levels, 1024 samples), three blocks 2202 us; 1024 x 512, 3 levels, 128 samples 76 and 92 us.  Source rows
 // staged in shared memory for levels 1 and 2 took 2020 us for the first and 229 us for the second: a row is
 // staged for too few samples unless the lobe is narrow and the count high.
-template <bool INT_SHIFT>
-__global__ void __launch_bounds__(kPrefilterThreads, 2)
+template <bool INT_SHIFT, int THREADS>
+__global__ void __launch_bounds__(THREADS, 512 / THREADS)
     k_prefilter(const __grid_constant__ MapDev src, const __grid_constant__ ChainDev ch, int N, int seg) {
   griddep_launch_dependents();
-  prefilter_segment<INT_SHIFT>(src, ch, N, seg);
+  prefilter_segment<INT_SHIFT, THREADS>(src, ch, N, seg);
   complete_in_order();
 }
 
@@ -1034,7 +1041,8 @@ static epbr_status launch_prefilter(const epbr_env* env, int N, const epbr_ibl* 
   if (ch.M > 1) {
     bool int_shift = true;
     for (int m = 1; m < ch.M; ++m) int_shift = int_shift && W0 % ch.W[m] == 0;
-    int seg = kPrefilterSeg;
+    const bool wide = int_shift && ch.W[1] >= kPrefilterWideMin && ch.W[1] <= kPrefilterWideMax && N >= kPrefilterWideSamples;
+    int seg = wide ? 2 * kPrefilterSeg : kPrefilterSeg;
     unsigned most = 0;
     for (;; seg /= 2) {
       long long blocks = 0;
@@ -1048,14 +1056,15 @@ static epbr_status launch_prefilter(const epbr_env* env, int N, const epbr_ibl* 
     }
     constexpr size_t kSampleBytes = sizeof(float4) + sizeof(int2) + sizeof(unsigned short);
     const size_t smem = (size_t)N * kSampleBytes;
-    void (*k)(const MapDev, const ChainDev, int, int) = int_shift ? k_prefilter<true> : k_prefilter<false>;
+    void (*k)(const MapDev, const ChainDev, int, int) = wide ? k_prefilter<true, 512> : (int_shift ? k_prefilter<true, 256> : k_prefilter<false, 256>);
     // for every count: without it the 48 KB limit also covers the kernel's static 6.3 KB
     if ((st = allow_shared(k, kPrefilterMaxSamples * kSampleBytes, "prefilter"))) return st;
     // a small shared-memory carve-out leaves most of the SM's 256 KB to L1, which holds the source rows the
     // resident blocks read (two rows of up to 16 KB per block); 40% (100 KB) holds two blocks of up to 1600
-    // samples: levels of a 2048 x 1024 environment at 50% 2101 us, at 40% 2060, at 25% (one block) 2321
-    cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 40);  // a hint; failure is harmless
-    if ((st = launched(launch_kernel(k, dim3(most, (unsigned)(ch.M - 1)), dim3(kPrefilterThreads), smem, s, early, src,
+    // samples, 58% (132 KB) two of any count: levels of a 2048 x 1024 environment at 50% 2101 us, at 40% 2060,
+    // at 25% (one block) 2321
+    cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, !wide && N > 1600 ? 58 : 40);  // a hint; failure is harmless
+    if ((st = launched(launch_kernel(k, dim3(most, (unsigned)(ch.M - 1)), dim3(wide ? 512 : 256), smem, s, early, src,
                                      ch, N, seg),
                        "k_prefilter")))
       return st;
