@@ -439,7 +439,8 @@ typedef struct epbr_surfels {
 } epbr_surfels;
 
 /* Device workspace epbr_surfel_gbuffer needs: 40 B per pixel, 4 B per pixel column and row, 96 B
- * and 8 B per surfel (list entries of the cells it covers, pixel box), each part 256-byte aligned. */
+ * and 8 B per surfel (list entries of the cells it covers, pixel box), each part 256-byte aligned; the
+ * pixels' share holds the cells' counters and the tiles whose lists are shared out. */
 epbr_status epbr_surfel_workspace_size(int32_t num_surfels, int32_t width, int32_t height, size_t* bytes);
 
 /* Writes the FP32 G-buffer `out` (rt[0] albedo + metal, rt[1] normal + rough, rt[3] eye depth;

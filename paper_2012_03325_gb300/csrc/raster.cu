@@ -193,10 +193,9 @@ struct RasterQueue {
 
 // Bound by instruction issue: about 600 warp instructions per 32 triangles and view (three vertex
 // transforms, the box, the serial pixels; ncu: 0.76 per scheduler and cycle), so the edge functions
-// are 32-bit wherever they fit and a triangle that no pixel centre can hit stops at its box.  Before,
-// a set-up pass wrote every visible triangle's 64 bytes and item count, three scan kernels numbered
-// all box pixels and a coverage kernel found each run of eight of them by a binary search over the
-// triangles: 122 us for the 1080p pass, 1650 us for the 64 maps; now 62 us and 467 us.
+// are 32-bit wherever they fit and a triangle that no pixel centre can hit stops at its box.  62 us for
+// the 1080p pass, 460 us for the 64 maps; 122 and 1650 us with a set-up pass, scans over the item counts and a
+// search per run of box pixels.
 // blockIdx.y = the view: its set-ups follow the previous views' (set-up view * T + t), its image
 // starts at view * view_px.  Set-ups are stored for the resolve (DEPTH 0) and for the queued ones.
 template <int DEPTH>
