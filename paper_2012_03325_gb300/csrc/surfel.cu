@@ -246,7 +246,7 @@ __device__ __forceinline__ HeavyRule heavy_rule(const SurfelHeader* h, unsigned 
 }
 __device__ __forceinline__ bool heavy_shared(const SurfelHeader* h, unsigned warps) {
   const unsigned longest = __ldcg(&h->longest);
-  return longest > 0 && longest > heavy_rule(h, warps).trigger;
+  return longest > kHeavyTrigger && longest > heavy_rule(h, warps).trigger;
 }
 __device__ __forceinline__ SurfelHeavy* heavy_at(char* end, unsigned slot) { return (SurfelHeavy*)end - (slot + 1); }
 __device__ __forceinline__ unsigned heavy_room(const SurfelHeader* h, const unsigned* list, const char* end) {
