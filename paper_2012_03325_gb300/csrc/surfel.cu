@@ -157,18 +157,18 @@ constexpr int kSurfelLevels = 14;         // enough for 32768 rows: the last lev
 constexpr int kSurfelCells = 24;          // list entries per surfel: 96 bytes of workspace
 // Atomics on one counter, or on counters of one 128-byte line, follow each other at 0.7 and 0.2 ns: with many
 // surfels for the cells the counts, not the tiles, bound the pass.  1.2 M surfels over a 64 x 64 view take
-// 1828 us with dense counters and 687 us with a line for each; spreading them over 256 KB and 512 KB
-// instead of 128 KB gains nothing there.
+// 1828 us with dense counters and 687 us with a line for each.  Arrays of at most 2^16, 2^17, 2^18 or 2^19 words:
+// 1.2 M surfels in the middle tenth of a 640 x 480 view 1012, 846, 805, 781 us; 70,000 over all of it 92, 82,
+// 79, 85.
 constexpr int kSurfelSpread = 131072;
 
 struct SurfelGrid {
   int levels;
   int stride;                       // words from one cell's counter to the next
-  __device__ __forceinline__ int at(int k) const { return k * stride; }
-
   int most;                         // cells a surfel is listed in at most
   int nx[kSurfelLevels];            // cells per row of a level
   int first[kSurfelLevels + 1];     // its first cell
+  __device__ __forceinline__ int at(int k) const { return k * stride; }
 };
 
 // Packed box: x0 | y0 << 16, width | height << 16 (each at most 32768; width 0: not drawn).
